@@ -31,6 +31,8 @@ struct LineTables {
     int nw, R;         // column-solver warps per CTA and rows per warp
     int r0, r1;        // interior rows with constant factors (interior_rows)
     double k[5];       // their l1, l2, 1/u0, u1/u0, u2/u0
+    double march[3];   // marching solver: l1, l2, 1/u0 of the unbounded line
+    int reach;         // its restart distance in rows, 0: the operator decays too slowly for it
 };
 
 }  // namespace chg

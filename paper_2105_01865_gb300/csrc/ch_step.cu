@@ -17,6 +17,7 @@
 #include "ch_explicit2.cuh"
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
+#include "ch_march.cuh"
 #include "line_tables.h"
 
 using namespace chg;
@@ -536,10 +537,178 @@ bool multi_line_any(const ch_handle* h, int l, int dir) {
     }
 }
 
+// Which form solves the lines of dir.  Measured per launch (us, launch gap
+// included; old: the scan solvers) on boxes nx x ny x nz, x / y / z:
+//   FP32  256 x 256 x 1    old  8.3 14.2  -    tile16  8.4  8.9  -    march 10.4 12.5  -
+//         96^3             old 10.3 12.4 10.7  tile16  8.6  8.6 10.5  march  8.3 10.1 11.2
+//         128^3            old 12.4 12.4 14.4  tile16 11.6 11.7 12.6  march 10.0 10.3 11.5
+//         256 x 256 x 128  old 29.0 39.8 30.0  tile16 26.7 25.2 33.0  march 16.4 16.4 24.9
+//         211 x 157 x 93   old 18.9 33.1 29.9  tile32 14.6 16.5 16.7  march 18.4 18.5 22.5
+//         500^3            old  311  356  390                         march  177  170  343
+//         1024 x 1024 x 512  old 1280 1420 1390                       march  663  648 1060
+//         1000 x 100 x 60, x only: old 26.4, march 36.9 (188 warps of 1000 rows)
+//   FP64  128^3            old  140  111  121  tile32   73   76   86  march  104  113  136
+//         256 x 256 x 128  old  382  444  369  tile32  218  217  266  march  258  281  359
+// So: the scan solvers where the operator decays too slowly, the restart is
+// longer than the line, or the line is short (whole steps with u = 0: FP32 64^3
+// old 59 us, new 70; 80^3 84 and 78; 128^3 113 and 92; FP64 64^3 471 and 436).  FP64, bound by its arithmetic, takes the form with the fewest
+// restarts, 32 rows a warp, where the line fits.  FP32 streams (march) once
+// 32-line groups outnumber the SMs two to one; fewer take 16 rows a warp, to
+// have warps enough; lines without 16-byte alignment, whose copies cost the
+// streaming warp an instruction an element, take 32 rows a warp up to 8 groups
+// an SM.  Long lines in few groups stay with the scans.
+enum LineForm { kLineScan, kLineTile16, kLineTile32, kLineMarch };
+template <typename T>
+LineForm line_form(const ch_handle* h, int l, int dir) {
+    const LineTables& lt = h->lines[dir][l];
+    const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
+    if (!lt.reach || lt.n < (sizeof(T) == 4 ? 65 : 64) || lt.reach > lt.n) return kLineScan;
+    const int64_t groups = dir == 0 ? (ny * nz + 31) / 32 : dir == 1 ? (nx + 31) / 32 * nz : (nx * ny + 31) / 32;
+    const int64_t row = dir == 2 ? nx * ny : nx;
+    const bool fits32 = tile_warps<32>(lt.n, lt.reach) <= tile_max_warps<32>() &&
+                        std::max(tile_yz_bytes<T, 32>(tile_warps<32>(lt.n, lt.reach)),
+                                 tile_x_bytes<T, 32>(tile_warps<32>(lt.n, lt.reach))) <= kMaxSmem;
+    if (sizeof(T) == 8) return fits32 ? kLineTile32 : groups >= 2 * 152 ? kLineMarch : kLineScan;
+    if (row % 4 != 0 && fits32 && groups <= 8 * 152) return kLineTile32;
+    if (groups <= 2 * 152 && tile_warps<16>(lt.n, lt.reach) <= tile_max_warps<16>()) return kLineTile16;
+    return groups >= 2 * 152 ? kLineMarch : kLineScan;
+}
+
+// Two columns per thread (paired FP32 arithmetic, 256-byte rows) while that
+// leaves 40 warps an SM: 1024 x 1024 x 512, y 651 against 667 us, z 1060
+// against 1100; on 256 x 256 x 128 one column is better, z 24.8 against 26.9.
+constexpr int64_t kMarchWide = 152 * 40;
+template <typename T>
+MarchCoef<T> march_coef(const ch_handle* h, int l, int dir) {
+    const LineTables& lt = h->lines[dir][l];
+    return {(T)-lt.march[0], (T)-lt.march[1], (T)lt.march[2], lt.n, h->p.bc[dir], lt.reach,
+            (lt.reach + MarchShape<T>::B - 1) / MarchShape<T>::B};
+}
+
+template <typename T, int V, int VL>
+int launch_march_yz(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+    const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
+    const MarchCoef<T> k = march_coef<T>(h, l, dir);
+    const size_t smem = march_yz_bytes<T, V>(k.kb);
+    const int64_t ncol = dir == 1 ? nx : nx * ny, ls = ncol, xg = (ncol + 32 * V - 1) / (32 * V);
+    const dim3 grid((unsigned)(xg * (dir == 1 ? nz : 1)));
+    if (Cupd)
+        launch_k(h->stream, ch_march_yz<T, V, VL, true>, grid, dim3(32), smem, (const T*)r, r, Cupd, (int)ncol, (int)xg,
+                 nx * ny, ls, k, h->status);
+    else
+        launch_k(h->stream, ch_march_yz<T, V, VL, false>, grid, dim3(32), smem, (const T*)r, r, (T*)nullptr, (int)ncol,
+                 (int)xg, nx * ny, ls, k, h->status);
+    CHG_CUDA(h, cudaGetLastError());
+    return CH_OK;
+}
+
+// Whole lines in shared memory, R rows per warp (ch_march.cuh).
+template <typename T, int R>
+int launch_tile(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+    const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
+    const MarchCoef<T> k = march_coef<T>(h, l, dir);
+    const int warps = tile_warps<R>(k.n, k.reach);
+    const dim3 block((unsigned)warps * 32);
+    if (dir == 0) {
+        launch_k(h->stream, ch_tile_x<T, R>, dim3((unsigned)((ny * nz + 31) / 32)), block, tile_x_bytes<T, R>(warps),
+                 (const T*)r, r, ny * nz, k);
+        CHG_CUDA(h, cudaGetLastError());
+        return CH_OK;
+    }
+    const size_t smem = tile_yz_bytes<T, R>(warps);
+    const int64_t ncol = dir == 1 ? nx : nx * ny, ls = ncol, xg = (ncol + 31) / 32;
+    const dim3 grid((unsigned)(xg * (dir == 1 ? nz : 1)));
+    constexpr int VEC = 16 / (int)sizeof(T);
+    auto go = [&](auto vlc) {
+        constexpr int VL = decltype(vlc)::value;
+        if (Cupd)
+            launch_k(h->stream, ch_tile_yz<T, R, VL, true>, grid, block, smem, (const T*)r, r, Cupd, (int)ncol, (int)xg,
+                     nx * ny, ls, k, h->status);
+        else
+            launch_k(h->stream, ch_tile_yz<T, R, VL, false>, grid, block, smem, (const T*)r, r, (T*)nullptr, (int)ncol,
+                     (int)xg, nx * ny, ls, k, h->status);
+    };
+    if (ncol % VEC == 0) go(std::integral_constant<int, VEC>{});
+    else go(std::integral_constant<int, 1>{});
+    CHG_CUDA(h, cudaGetLastError());
+    return CH_OK;
+}
+
+template <typename T>
+int launch_march(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+    const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
+    if (dir == 0) {
+        const MarchCoef<T> k = march_coef<T>(h, l, dir);
+        launch_k(h->stream, ch_march_x<T>, dim3((unsigned)((ny * nz + 31) / 32)), dim3(32), march_x_bytes<T>(k.kb),
+                 (const T*)r, r, ny * nz, k);
+        CHG_CUDA(h, cudaGetLastError());
+        return CH_OK;
+    }
+    constexpr int VEC = 16 / (int)sizeof(T);
+    const int64_t row = dir == 1 ? nx : nx * ny;  // columns of a row: its alignment
+    if constexpr (sizeof(T) == 4) {
+        const int64_t wide = (row + 63) / 64 * (dir == 1 ? nz : 1);
+        if (row % VEC == 0 && wide >= kMarchWide) return launch_march_yz<T, 2, VEC>(h, l, dir, r, Cupd);
+    }
+    return row % VEC == 0 ? launch_march_yz<T, 1, VEC>(h, l, dir, r, Cupd) : launch_march_yz<T, 1, 1>(h, l, dir, r, Cupd);
+}
+
+template <typename T, int V, int VL>
+int set_attrs_march_yz(ch_handle* h) {
+    const int shm = (int)march_yz_bytes<T, V>(march_max_kb<T>());
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_yz<T, V, VL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_yz<T, V, VL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_yz<T, V, VL, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_yz<T, V, VL, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    return CH_OK;
+}
+
+template <typename T, int R>
+int set_attrs_tile(ch_handle* h) {
+    constexpr int VEC = 16 / (int)sizeof(T);
+    const int yz = (int)std::min(tile_yz_bytes<T, R>(tile_max_warps<R>()), kMaxSmem), x = (int)std::min(tile_x_bytes<T, R>(tile_max_warps<R>()), kMaxSmem);
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_tile_x<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, x));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_tile_yz<T, R, VEC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, yz));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_tile_yz<T, R, VEC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, yz));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_tile_yz<T, R, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, yz));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_tile_yz<T, R, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, yz));
+    return CH_OK;
+}
+
+template <typename T>
+int set_attrs_march(ch_handle* h) {
+    constexpr int VEC = 16 / (int)sizeof(T);
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_x<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)march_x_bytes<T>(march_max_kb<T>())));
+    CHG_CUDA(h, cudaFuncSetAttribute(ch_march_x<T>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    int rc = set_attrs_march_yz<T, 1, VEC>(h);
+    if (rc == CH_OK) rc = set_attrs_march_yz<T, 1, 1>(h);
+    if constexpr (sizeof(T) == 4) {
+        if (rc == CH_OK) rc = set_attrs_march_yz<T, 2, VEC>(h);
+    }
+    if constexpr (sizeof(T) == 4)
+        if (rc == CH_OK) rc = set_attrs_tile<T, 16>(h);
+    if (rc == CH_OK) rc = set_attrs_tile<T, 32>(h);
+    return rc;
+}
+
 template <typename T>
 int launch_solve(ch_handle* h, int l, int dir, T* r, T* Cupd, cudaEvent_t ev_after) {
+    int rc = -1;
+    switch (line_form<T>(h, l, dir)) {
+        case kLineMarch: rc = launch_march<T>(h, l, dir, r, Cupd); break;
+        case kLineTile32: rc = launch_tile<T, 32>(h, l, dir, r, Cupd); break;
+        case kLineTile16:
+            if constexpr (sizeof(T) == 4) rc = launch_tile<T, 16>(h, l, dir, r, Cupd);
+            break;
+        case kLineScan: break;
+    }
+    if (rc >= 0) {
+        if (rc == CH_OK && ev_after) CHG_CUDA(h, cudaEventRecord(ev_after, h->stream));
+        return rc;
+    }
     if (dir > 0 && !multi_line_any<T>(h, l, dir)) {
-        const int rc = launch_cols<T>(h, l, dir, r, Cupd);
+        rc = launch_cols<T>(h, l, dir, r, Cupd);
         if (rc >= 0) {
             if (rc == CH_OK && ev_after) CHG_CUDA(h, cudaEventRecord(ev_after, h->stream));
             return rc;
@@ -712,6 +881,7 @@ int set_smem_attrs(ch_handle* h) {
     if (rc == CH_OK) rc = set_attrs_m<T, 32>(h);
     if constexpr (sizeof(T) == 4)
         if (rc == CH_OK) rc = set_attrs_cols2_all<T>(h);
+    if (rc == CH_OK) rc = set_attrs_march<T>(h);
     return rc;
 }
 
@@ -912,6 +1082,12 @@ int ch_create(const ch_params* p, void* C, void* work, size_t work_bytes, void* 
                 lt.r0 = I.r0;
                 lt.r1 = I.r1;
                 for (int m = 0; m < 5; ++m) lt.k[m] = I.k[m];
+                const MarchFactors mf = h->esz == 8 ? march_factors<double>(ck, kMarchMaxReach, std::ldexp(1.0, -64))
+                                                    : march_factors<float>(ck, kMarchMaxReach, std::ldexp(1.0, -36));
+                lt.march[0] = mf.l1;
+                lt.march[1] = mf.l2;
+                lt.march[2] = mf.dinv;
+                lt.reach = mf.reach;
                 total += align_up(all.back().size() * h->esz);
                 // y and z lines also get column-solver tables when they fit
                 int nw = 0, R = 0;

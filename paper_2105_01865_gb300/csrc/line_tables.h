@@ -6,7 +6,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstddef>
+#include <limits>
 #include <tuple>
 #include <utility>
 #include <vector>
@@ -244,6 +246,77 @@ Interior interior_rows(const LineFactors& F) {
     I.k[3] = F.u1s[mid];
     I.k[4] = F.u2s[mid];
     return I;
+}
+
+// Constant factors of the operator on an unbounded line (ch_march.cuh):
+// 1 + ck [1,-4,6,-4,1] = u0 (1 + l1 S^-1 + l2 S^-2)(1 + l1 S + l2 S^2), S the
+// shift by one row.  Its symbol z^2 + ck (1 - z)^4 = 0 gives (1 - z)^2 =
+// +-i z / sqrt(ck); the pair of roots inside the unit circle, z and its
+// conjugate, makes both recurrences decay: l1 = -2 Re z, l2 = |z|^2 and
+// u0 = ck / l2.  z is taken as the reciprocal of the outer root, which has no
+// cancellation for small ck.  reach: the restart distance, the smallest multiple
+// of 8 rows whose 2 x 2 transfer matrix has no entry over tol; 0 if over
+// max_reach.
+//
+// The factors are returned rounded to T.  Rounded one by one they would solve
+// with an operator that is off by up to 2^-24 / |1 - z|^2 where it varies
+// slowly along the line (1 + l1 + l2 = |1 - z|^2 is small for large ck).  Of the
+// values a few units in the last place about l1 and l2, with 1/u0 following
+// from a unit response to a constant line, those are taken whose response
+// over all wave numbers is nearest to the exact one.
+struct MarchFactors {
+    double l1 = 0, l2 = 0, dinv = 0;
+    int reach = 0;
+};
+
+template <typename T>
+MarchFactors march_factors(double ck, int max_reach, double tol) {
+    MarchFactors f;
+    const std::complex<double> w(2.0, 1.0 / std::sqrt(ck)), q = std::sqrt(w * w - 4.0);
+    const std::complex<double> big = std::abs(w + q) > std::abs(w - q) ? w + q : w - q, z = 2.0 / big;
+    f.l1 = -2.0 * z.real();
+    f.l2 = std::norm(z);
+    f.dinv = f.l2 / ck;
+    if (!std::isfinite(f.l1) || !std::isfinite(f.dinv) || !(f.l2 > 0.0) || !(f.dinv > 0.0)) return f;
+    double m[4] = {1, 0, 0, 1};  // [[-l1, -l2], [1, 0]]^rows
+    for (int rows = 8; rows <= max_reach && !f.reach; rows += 8) {
+        for (int i = 0; i < 8; ++i) {
+            const double a = -f.l1 * m[0] - f.l2 * m[2], b = -f.l1 * m[1] - f.l2 * m[3];
+            m[2] = m[0]; m[3] = m[1];
+            m[0] = a; m[1] = b;
+        }
+        double big_entry = 0.0;
+        for (double e : m) big_entry = std::max(big_entry, std::fabs(e));
+        if (big_entry <= tol) f.reach = rows;
+    }
+    if (sizeof(T) == sizeof(double)) return f;  // rounded to FP64 as computed
+    auto step = [](T v, int u) {  // u units in the last place from v
+        for (; u > 0; --u) v = std::nextafter(v, std::numeric_limits<T>::infinity());
+        for (; u < 0; ++u) v = std::nextafter(v, -std::numeric_limits<T>::infinity());
+        return v;
+    };
+    constexpr int kWaves = 24;
+    double best = -1.0;
+    MarchFactors r = f;
+    for (int u1 = -1; u1 <= 1; ++u1)
+        for (int u2 = -4; u2 <= 4; ++u2) {
+            const double l1 = step((T)f.l1, u1), l2 = step((T)f.l2, u2);
+            const double dc = 1.0 + l1 + l2, dinv = (T)(dc * dc);
+            double off = 0.0;
+            for (int p = 0; p < kWaves; ++p) {
+                const double t = 3.14159265358979323846 * p * p / ((kWaves - 1) * (kWaves - 1));  // finer where it is slow
+                const double re = 1.0 + l1 * std::cos(t) + l2 * std::cos(2 * t), im = l1 * std::sin(t) + l2 * std::sin(2 * t);
+                const double s2 = 2.0 - 2.0 * std::cos(t);
+                off = std::max(off, std::fabs(dinv * (1.0 + ck * s2 * s2) / (re * re + im * im) - 1.0));
+            }
+            if (best < 0.0 || off < best) {
+                best = off;
+                r.l1 = l1;
+                r.l2 = l2;
+                r.dinv = dinv;
+            }
+        }
+    return r;
 }
 
 // Rows per lane of the warp-scan solver: the smallest power of two M with

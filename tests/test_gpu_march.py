@@ -1,0 +1,54 @@
+"""GPU tests of the marching line solver: one u = 0 step against the oracle
+where its blocks, restarts and ghost rows can go wrong (line lengths about the
+block sizes, lines shorter than the restart distance, every wall type, every
+copy width), for operators of each restart distance and for one that decays
+too slowly and takes the scan solvers."""
+import numpy as np
+import pytest
+
+from oracle import ch_oracle as co
+from paper_2105_01865_gb300 import inputs
+
+from _parity import assert_parity
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+P, N, D = co.PERIODIC, co.NOFLUX, co.DIRICHLET
+# (nz, ny, nx): lines of 5 to 3 blocks and a remainder; nx odd, even, a multiple of 4
+SHAPES = [(5, 6, 7), (31, 33, 32), (64, 65, 34), (33, 5, 97), (100, 31, 66), (7, 129, 36), (129, 8, 5), (6, 40, 160)]
+BCS = [(P, P, P), (N, N, N), (P, N, D), (N, P, P)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2105_01865_gb300 import build, capi
+    build.build()
+    capi.load()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("shape", SHAPES)
+# ck of the first substep: restart distances of 1, 2 and 3 blocks, and the scan solvers
+@pytest.mark.parametrize("ck", [0.02, 1.2, 12.0, 400.0])
+def test_one_step_matches_oracle(shape, ck, prec):
+    from paper_2105_01865_gb300.solver import Solver
+    nz, ny, nx = shape
+    h, cn, pe = 1.0 / 32, 0.75 / 32, 100.0
+    bc = BCS[(SHAPES.index(shape) + int(ck)) % len(BCS)]
+    dt = ck / (8.0 / 15.0 / pe / 2.0 * 4.0 * cn ** 2 / h ** 4)
+    rng = np.random.default_rng(nx)
+    C0 = inputs.drops_field(shape, h, bc, [(nx * h / 2, ny * h / 3, nz * h / 2)], [0.3 * min(shape) * h], cn)
+    C0 = C0 + 0.05 * rng.standard_normal(shape)
+    if prec == "f32":
+        C0 = C0.astype(np.float32).astype(np.float64)
+    s = Solver(shape, h, bc, cn, pe, dt, C0, precision=prec)
+    s.step(1)
+    got = s.field()
+    s.close()
+    ref = co.step(C0, None, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=dt, bc=bc), 1)
+    # backward-stable solves: a few roundings times the condition number of (I + ck [1,-4,6,-4,1])
+    assert_parity(got, ref, 8 * (1 + 16 * ck) * 2.0 ** (-53 if prec == "f64" else -24), f"march {shape} {bc} ck={ck} {prec}")
