@@ -32,57 +32,117 @@ struct AdjArgs {
 };
 
 template <typename T>
-__device__ __forceinline__ T at(const T* f, int i, int j, int k, const AdjArgs<T>& a) {
-    return f[((int64_t)bc_index(k, a.nz, a.bcz) * a.ny + bc_index(j, a.ny, a.bcy)) * a.nx + bc_index(i, a.nx, a.bcx)];
-}
+__device__ __forceinline__ T psi_prime_t(T c) { return c * (c * (c - T(1.5)) + T(0.5)); }
 
+// Sum of products for dL/dM.  FP64 fields multiply and add in FP64.  FP32
+// fields keep a double-float pair: the product's rounding error comes exactly
+// out of one fused multiply-add, the sum's out of TwoSum, so a thread's partial
+// sum is good to about 2^-48 of its terms without FP64 arithmetic, which would
+// bound the kernel (8 multiply-adds and 9 conversions a cell at 1/64 of the
+// FP32 rate).
 template <typename T>
-__device__ __forceinline__ T fourth(const T* f, int i, int j, int k, int d, const AdjArgs<T>& a) {
-    const int di = d == 0, dj = d == 1, dk = d == 2;
-    const T c = f[((int64_t)k * a.ny + j) * a.nx + i];
-    const T m1 = at(f, i - di, j - dj, k - dk, a), p1 = at(f, i + di, j + dj, k + dk, a);
-    const T m2 = at(f, i - 2 * di, j - 2 * dj, k - 2 * dk, a), p2 = at(f, i + 2 * di, j + 2 * dj, k + 2 * dk, a);
+struct AdjDot {
+    T s = T(0);
+    __device__ __forceinline__ void add(T a, T b) { s += a * b; }
+    __device__ __forceinline__ double total() const { return s; }
+};
+template <>
+struct AdjDot<float> {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float x = __fmul_rn(a, b);
+        const float xe = __fmaf_rn(a, b, -x);
+        const float t = __fadd_rn(s, x);
+        const float bp = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(x, bp)), xe));
+        s = t;
+    }
+    __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+};
+
+// [1,-4,6,-4,1] of five neighbours along one direction, as differences
+template <typename T>
+__device__ __forceinline__ T fourth(T m2, T m1, T c, T p1, T p2) {
     const T da = m1 - c, db = p1 - c;
     return ((m2 - m1) - da) + ((p2 - p1) - db) - T(2) * (da + db);
 }
 
-template <typename T>
-__device__ __forceinline__ T psi_prime_t(T c) { return c * (c * (c - T(1.5)) + T(0.5)); }
-
-// One thread per cell: the reverse substep map above, in the field precision,
-// with the dL/dM terms accumulated per block in FP64.
+// The reverse substep map above, in the field precision.  A thread marches
+// kAdjZ planes of its column: its z-neighbours stay in registers, and the
+// in-plane ones are read through offsets found once, so a cell costs 27 loads
+// that neighbouring threads share in L1.  Bound by those loads.  One thread a
+// cell, with every neighbour's index reduced modulo the box, took 356 us on
+// 128^3 (FP32); this form 50.
+constexpr int kAdjZ = 8;
 template <typename T>
 __global__ void __launch_bounds__(kAThreadsX * kAThreadsY)
-adj_substep(const T* C, const T* lam_r, const T* lamH_in, const T* lamC_in, const T* s0, const T* s1, const T* s2,
-            T* lamC_out, T* lamHp_out, double* partials, AdjArgs<T> a) {
+adj_substep(const T* __restrict__ C, const T* __restrict__ lam_r, const T* __restrict__ lamH_in,
+            const T* __restrict__ lamC_in, const T* __restrict__ s0, const T* __restrict__ s1,
+            const T* __restrict__ s2, T* __restrict__ lamC_out, T* __restrict__ lamHp_out, double* partials,
+            AdjArgs<T> a) {
     const int i = blockIdx.x * kAThreadsX + threadIdx.x;
     const int j = blockIdx.y * kAThreadsY + threadIdx.y;
-    const int k = blockIdx.z;
+    const int k0 = blockIdx.z * kAdjZ, k1 = min(k0 + kAdjZ, a.nz);
     double dm = 0.0;
     if (i < a.nx && j < a.ny) {
-        const int64_t e = ((int64_t)k * a.ny + j) * a.nx + i;
+        // in-plane neighbours of (i, j), as offsets from it
+        const int64_t plane = (int64_t)a.nx * a.ny, ij = (int64_t)j * a.nx + i;
+        const int xm1 = bc_near(i - 1, a.nx, a.bcx) - i, xp1 = bc_near(i + 1, a.nx, a.bcx) - i;
+        const int xm2 = bc_near(i - 2, a.nx, a.bcx) - i, xp2 = bc_near(i + 2, a.nx, a.bcx) - i;
+        const int ym1 = (bc_near(j - 1, a.ny, a.bcy) - j) * a.nx, yp1 = (bc_near(j + 1, a.ny, a.bcy) - j) * a.nx;
+        const int ym2 = (bc_near(j - 2, a.ny, a.bcy) - j) * a.nx, yp2 = (bc_near(j + 2, a.ny, a.bcy) - j) * a.nx;
+        auto zoff = [&](int k) { return bc_near(k, a.nz, a.bcz) * plane + ij; };
         const T dtg = T(a.dt * a.gamma), mob = T(a.mob), inv_h2 = T(a.inv_h2), kap = T(a.kappa);
-        auto lamH = [&](int ii, int jj, int kk) { return dtg * at(lam_r, ii, jj, kk, a) + at(lamH_in, ii, jj, kk, a); };
-        auto psi_at = [&](int ii, int jj, int kk) { return psi_prime_t(at(C, ii, jj, kk, a)); };
-        const T lh0 = lamH(i, j, k);
-        const T lap_lh = ((lamH(i - 1, j, k) - lh0) + (lamH(i + 1, j, k) - lh0) + (lamH(i, j - 1, k) - lh0) +
-                          (lamH(i, j + 1, k) - lh0) + (lamH(i, j, k - 1) - lh0) + (lamH(i, j, k + 1) - lh0)) *
-                         inv_h2;
-        const T p0 = psi_at(i, j, k);
-        const T lap_psi = ((psi_at(i - 1, j, k) - p0) + (psi_at(i + 1, j, k) - p0) + (psi_at(i, j - 1, k) - p0) +
-                           (psi_at(i, j + 1, k) - p0) + (psi_at(i, j, k - 1) - p0) + (psi_at(i, j, k + 1) - p0)) *
-                          inv_h2;
-        const T A_lr[3] = {kap * fourth(lam_r, i, j, k, 0, a), kap * fourth(lam_r, i, j, k, 1, a),
-                           kap * fourth(lam_r, i, j, k, 2, a)};
-        const T A_C = kap * (fourth(C, i, j, k, 0, a) + fourth(C, i, j, k, 1, a) + fourth(C, i, j, k, 2, a));
-        const T c = C[e];
-        const T ppp = (T(3) * c - T(3)) * c + T(0.5);
-        const T adt = T(a.alpha * a.dt);
-        lamC_out[e] = lamC_in[e] - adt * mob * ((A_lr[0] + A_lr[1]) + A_lr[2]) + ppp * mob * lap_lh;
-        lamHp_out[e] = T(a.dt * a.rho) * lam_r[e];
-        dm = (double)lh0 * (double)lap_psi - a.alpha * a.dt * (double)lam_r[e] * (double)A_C -
-             0.5 * a.alpha * a.dt *
-                 ((double)A_lr[0] * (double)s0[e] + (double)A_lr[1] * (double)s1[e] + (double)A_lr[2] * (double)s2[e]);
+        const T adt = T(a.alpha * a.dt), dtr = T(a.dt * a.rho);
+        // q[m] = row k - 2 + m of C and lam_r; lam_H' of this substep one row down and at k
+        T qc[5], ql[5];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            qc[m] = C[zoff(k0 - 2 + m)];
+            ql[m] = lam_r[zoff(k0 - 2 + m)];
+        }
+        T hm = lamH_in[zoff(k0 - 1)], hc = lamH_in[zoff(k0)];
+        AdjDot<T> d1, d2;  // <lam_H, lap psi'> and <lam_r, A C> + sum_d <A_d lam_r, s_d> / 2
+        for (int k = k0; k < k1; ++k) {
+            const int64_t e = k * plane + ij, z2 = zoff(k + 2);
+            qc[4] = C[z2];
+            ql[4] = lam_r[z2];
+            const T hp = lamH_in[zoff(k + 1)];
+            const T *pc = C + e, *pl = lam_r + e, *ph = lamH_in + e;
+            const T c = qc[2], lr = ql[2];
+            const T cxm = pc[xm1], cxp = pc[xp1], cym = pc[ym1], cyp = pc[yp1];
+            const T lxm = pl[xm1], lxp = pl[xp1], lym = pl[ym1], lyp = pl[yp1];
+            const T lh0 = dtg * lr + hc;
+            const T lap_lh = (((dtg * lxm + ph[xm1]) - lh0) + ((dtg * lxp + ph[xp1]) - lh0) +
+                              ((dtg * lym + ph[ym1]) - lh0) + ((dtg * lyp + ph[yp1]) - lh0) +
+                              ((dtg * ql[1] + hm) - lh0) + ((dtg * ql[3] + hp) - lh0)) *
+                             inv_h2;
+            const T p0 = psi_prime_t(c);
+            const T lap_psi = ((psi_prime_t(cxm) - p0) + (psi_prime_t(cxp) - p0) + (psi_prime_t(cym) - p0) +
+                               (psi_prime_t(cyp) - p0) + (psi_prime_t(qc[1]) - p0) + (psi_prime_t(qc[3]) - p0)) *
+                              inv_h2;
+            const T A_lr[3] = {kap * fourth(pl[xm2], lxm, lr, lxp, pl[xp2]),
+                               kap * fourth(pl[ym2], lym, lr, lyp, pl[yp2]),
+                               kap * fourth(ql[0], ql[1], lr, ql[3], ql[4])};
+            const T A_C = kap * (fourth(pc[xm2], cxm, c, cxp, pc[xp2]) + fourth(pc[ym2], cym, c, cyp, pc[yp2]) +
+                                 fourth(qc[0], qc[1], c, qc[3], qc[4]));
+            const T ppp = (T(3) * c - T(3)) * c + T(0.5);
+            lamC_out[e] = lamC_in[e] - adt * mob * ((A_lr[0] + A_lr[1]) + A_lr[2]) + ppp * mob * lap_lh;
+            lamHp_out[e] = dtr * lr;
+            d1.add(lh0, lap_psi);
+            d2.add(lr, A_C);
+            d2.add(T(0.5) * A_lr[0], s0[e]);
+            d2.add(T(0.5) * A_lr[1], s1[e]);
+            d2.add(T(0.5) * A_lr[2], s2[e]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                qc[m] = qc[m + 1];
+                ql[m] = ql[m + 1];
+            }
+            hm = hc;
+            hc = hp;
+        }
+        dm = d1.total() - a.alpha * a.dt * d2.total();
     }
     __shared__ double ws[kAThreadsX * kAThreadsY / 32];
     for (int o = 16; o > 0; o >>= 1) dm += __shfl_xor_sync(0xffffffffu, dm, o);
@@ -122,7 +182,7 @@ AdjLayout adj_layout(const ch_handle* h, int64_t nsteps, int64_t K) {
     L.nck = (size_t)((nsteps + K - 1) / K);
     L.K = (size_t)std::min(K, nsteps);
     const size_t nblocks = (size_t)((h->n[0] + kAThreadsX - 1) / kAThreadsX) *
-                           ((h->n[1] + kAThreadsY - 1) / kAThreadsY) * h->n[2];
+                           ((h->n[1] + kAThreadsY - 1) / kAThreadsY) * ((h->n[2] + kAdjZ - 1) / kAdjZ);
     L.total = (L.nck + L.K + 15) * L.field + a256(nblocks * sizeof(double)) + 256;
     return L;
 }
@@ -169,7 +229,7 @@ int ch_step_adjoint(ch_handle* h, const void* C0, int64_t nsteps, int64_t ckpt_e
     cudaStream_t st = h->stream;
     const ch_params& p = h->p;
     const int nx = (int)h->n[0], ny = (int)h->n[1], nz = (int)h->n[2];
-    dim3 grid((nx + kAThreadsX - 1) / kAThreadsX, (ny + kAThreadsY - 1) / kAThreadsY, nz);
+    dim3 grid((nx + kAThreadsX - 1) / kAThreadsX, (ny + kAThreadsY - 1) / kAThreadsY, (nz + kAdjZ - 1) / kAdjZ);
     dim3 block(kAThreadsX, kAThreadsY);
     const int64_t nblk = (int64_t)grid.x * grid.y * grid.z;
     auto cp = [&](void* dst, const void* src) {
@@ -202,17 +262,14 @@ int ch_step_adjoint(ch_handle* h, const void* C0, int64_t nsteps, int64_t ckpt_e
             for (int l = 0; l < 2 && rc == CH_OK; ++l) {
                 rc = launch_explicit_any(h, l, X[l], l ? Hs[l - 1] : nullptr, Hs[l], rtmp);
                 CHG_CUDA(h, cp(X[l + 1], X[l]));
-                for (int d = 0; d < 3 && rc == CH_OK; ++d) rc = launch_solve_any(h, l, d, rtmp, d == 2 ? X[l + 1] : nullptr);
+                for (int d = 0; d < 3 && rc == CH_OK; ++d)
+                    rc = launch_solve_any(h, l, d, rtmp, rtmp, d == 2 ? X[l + 1] : nullptr);
             }
             CHG_CUDA(h, cudaMemsetAsync(lamH, 0, fb, st));
             for (int l = 2; l >= 0 && rc == CH_OK; --l) {
                 rc = launch_explicit_any(h, l, X[l], l ? Hs[l - 1] : nullptr, Htmp, rtmp);
-                CHG_CUDA(h, cp(lamr, lamC));
-                for (int d = 0; d < 3 && rc == CH_OK; ++d) rc = launch_solve_any(h, l, d, lamr, nullptr);
-                for (int d = 0; d < 3 && rc == CH_OK; ++d) {
-                    CHG_CUDA(h, cp(sd[d], rtmp));
-                    rc = launch_solve_any(h, l, d, sd[d], nullptr);
-                }
+                for (int d = 0; d < 3 && rc == CH_OK; ++d) rc = launch_solve_any(h, l, d, d ? lamr : lamC, lamr, nullptr);
+                for (int d = 0; d < 3 && rc == CH_OK; ++d) rc = launch_solve_any(h, l, d, rtmp, sd[d], nullptr);
                 if (rc != CH_OK) break;
                 if (h->prec == CH_F64) {
                     AdjArgs<double> a{nx, ny, nz, p.bc[0], p.bc[1], p.bc[2], p.dt, kGamma[l], kRho[l], kGamma[l] + kRho[l],

@@ -104,7 +104,8 @@ inline int fail(ch_handle* h, int code, const char* fmt, ...) {
 
 // launchers shared with the adjoint (ch_step.cu), in the handle's precision
 int launch_explicit_any(ch_handle* h, int l, const void* C, const void* Hprev, void* Hout, void* r);
-int launch_solve_any(ch_handle* h, int l, int dir, void* a, void* Cupd);
+// the solution of src's lines into dst (which may be src), or added to Cupd
+int launch_solve_any(ch_handle* h, int l, int dir, const void* src, void* dst, void* Cupd);
 int launch_step_any(ch_handle* h, void* C);  // one full step of the field C (direct launches)
 // -div(uC) alone into Hout (the standard scheme's advection; ch_step.cu)
 int launch_advection_any(ch_handle* h, const void* C, void* Hout);

@@ -586,17 +586,17 @@ MarchCoef<T> march_coef(const ch_handle* h, int l, int dir) {
 }
 
 template <typename T, int V, int VL>
-int launch_march_yz(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+int launch_march_yz(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd) {
     const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
     const MarchCoef<T> k = march_coef<T>(h, l, dir);
     const size_t smem = march_yz_bytes<T, V>(k.kb);
     const int64_t ncol = dir == 1 ? nx : nx * ny, ls = ncol, xg = (ncol + 32 * V - 1) / (32 * V);
     const dim3 grid((unsigned)(xg * (dir == 1 ? nz : 1)));
     if (Cupd)
-        launch_k(h->stream, ch_march_yz<T, V, VL, true>, grid, dim3(32), smem, (const T*)r, r, Cupd, (int)ncol, (int)xg,
+        launch_k(h->stream, ch_march_yz<T, V, VL, true>, grid, dim3(32), smem, src, r, Cupd, (int)ncol, (int)xg,
                  nx * ny, ls, k, h->status);
     else
-        launch_k(h->stream, ch_march_yz<T, V, VL, false>, grid, dim3(32), smem, (const T*)r, r, (T*)nullptr, (int)ncol,
+        launch_k(h->stream, ch_march_yz<T, V, VL, false>, grid, dim3(32), smem, src, r, (T*)nullptr, (int)ncol,
                  (int)xg, nx * ny, ls, k, h->status);
     CHG_CUDA(h, cudaGetLastError());
     return CH_OK;
@@ -604,14 +604,14 @@ int launch_march_yz(ch_handle* h, int l, int dir, T* r, T* Cupd) {
 
 // Whole lines in shared memory, R rows per warp (ch_march.cuh).
 template <typename T, int R>
-int launch_tile(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+int launch_tile(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd) {
     const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
     const MarchCoef<T> k = march_coef<T>(h, l, dir);
     const int warps = tile_warps<R>(k.n, k.reach);
     const dim3 block((unsigned)warps * 32);
     if (dir == 0) {
         launch_k(h->stream, ch_tile_x<T, R>, dim3((unsigned)((ny * nz + 31) / 32)), block, tile_x_bytes<T, R>(warps),
-                 (const T*)r, r, ny * nz, k);
+                 src, r, ny * nz, k);
         CHG_CUDA(h, cudaGetLastError());
         return CH_OK;
     }
@@ -622,10 +622,10 @@ int launch_tile(ch_handle* h, int l, int dir, T* r, T* Cupd) {
     auto go = [&](auto vlc) {
         constexpr int VL = decltype(vlc)::value;
         if (Cupd)
-            launch_k(h->stream, ch_tile_yz<T, R, VL, true>, grid, block, smem, (const T*)r, r, Cupd, (int)ncol, (int)xg,
+            launch_k(h->stream, ch_tile_yz<T, R, VL, true>, grid, block, smem, src, r, Cupd, (int)ncol, (int)xg,
                      nx * ny, ls, k, h->status);
         else
-            launch_k(h->stream, ch_tile_yz<T, R, VL, false>, grid, block, smem, (const T*)r, r, (T*)nullptr, (int)ncol,
+            launch_k(h->stream, ch_tile_yz<T, R, VL, false>, grid, block, smem, src, r, (T*)nullptr, (int)ncol,
                      (int)xg, nx * ny, ls, k, h->status);
     };
     if (ncol % VEC == 0) go(std::integral_constant<int, VEC>{});
@@ -635,12 +635,12 @@ int launch_tile(ch_handle* h, int l, int dir, T* r, T* Cupd) {
 }
 
 template <typename T>
-int launch_march(ch_handle* h, int l, int dir, T* r, T* Cupd) {
+int launch_march(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd) {
     const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
     if (dir == 0) {
         const MarchCoef<T> k = march_coef<T>(h, l, dir);
         launch_k(h->stream, ch_march_x<T>, dim3((unsigned)((ny * nz + 31) / 32)), dim3(32), march_x_bytes<T>(k.kb),
-                 (const T*)r, r, ny * nz, k);
+                 src, r, ny * nz, k);
         CHG_CUDA(h, cudaGetLastError());
         return CH_OK;
     }
@@ -648,9 +648,9 @@ int launch_march(ch_handle* h, int l, int dir, T* r, T* Cupd) {
     const int64_t row = dir == 1 ? nx : nx * ny;  // columns of a row: its alignment
     if constexpr (sizeof(T) == 4) {
         const int64_t wide = (row + 63) / 64 * (dir == 1 ? nz : 1);
-        if (row % VEC == 0 && wide >= kMarchWide) return launch_march_yz<T, 2, VEC>(h, l, dir, r, Cupd);
+        if (row % VEC == 0 && wide >= kMarchWide) return launch_march_yz<T, 2, VEC>(h, l, dir, src, r, Cupd);
     }
-    return row % VEC == 0 ? launch_march_yz<T, 1, VEC>(h, l, dir, r, Cupd) : launch_march_yz<T, 1, 1>(h, l, dir, r, Cupd);
+    return row % VEC == 0 ? launch_march_yz<T, 1, VEC>(h, l, dir, src, r, Cupd) : launch_march_yz<T, 1, 1>(h, l, dir, src, r, Cupd);
 }
 
 template <typename T, int V, int VL>
@@ -693,13 +693,13 @@ int set_attrs_march(ch_handle* h) {
 }
 
 template <typename T>
-int launch_solve(ch_handle* h, int l, int dir, T* r, T* Cupd, cudaEvent_t ev_after) {
+int launch_solve(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd, cudaEvent_t ev_after) {
     int rc = -1;
     switch (line_form<T>(h, l, dir)) {
-        case kLineMarch: rc = launch_march<T>(h, l, dir, r, Cupd); break;
-        case kLineTile32: rc = launch_tile<T, 32>(h, l, dir, r, Cupd); break;
+        case kLineMarch: rc = launch_march<T>(h, l, dir, src, r, Cupd); break;
+        case kLineTile32: rc = launch_tile<T, 32>(h, l, dir, src, r, Cupd); break;
         case kLineTile16:
-            if constexpr (sizeof(T) == 4) rc = launch_tile<T, 16>(h, l, dir, r, Cupd);
+            if constexpr (sizeof(T) == 4) rc = launch_tile<T, 16>(h, l, dir, src, r, Cupd);
             break;
         case kLineScan: break;
     }
@@ -707,6 +707,8 @@ int launch_solve(ch_handle* h, int l, int dir, T* r, T* Cupd, cudaEvent_t ev_aft
         if (rc == CH_OK && ev_after) CHG_CUDA(h, cudaEventRecord(ev_after, h->stream));
         return rc;
     }
+    if (src != r)  // the scan solvers work in place
+        CHG_CUDA(h, cudaMemcpyAsync(r, src, (size_t)h->ncell * sizeof(T), cudaMemcpyDeviceToDevice, h->stream));
     if (dir > 0 && !multi_line_any<T>(h, l, dir)) {
         rc = launch_cols<T>(h, l, dir, r, Cupd);
         if (rc >= 0) {
@@ -864,7 +866,7 @@ int launch_substep(ch_handle* h, int l, cudaEvent_t* ev = nullptr) {
             if (ev) CHG_CUDA(h, cudaEventRecord(ev[4], h->stream));
             continue;
         }
-        rc = launch_solve<T>(h, l, dir, r, dir == 2 ? C : nullptr, ev ? ev[2 + dir] : nullptr);
+        rc = launch_solve<T>(h, l, dir, r, r, dir == 2 ? C : nullptr, ev ? ev[2 + dir] : nullptr);
         if (rc != CH_OK) return rc;
     }
     return CH_OK;
@@ -901,9 +903,10 @@ int launch_advection_any(ch_handle* h, const void* C, void* Hout) {
     return launch_explicit<float>(h, 0, (const float*)C, nullptr, (float*)Hout, nullptr, nullptr, true);
 }
 
-int launch_solve_any(ch_handle* h, int l, int dir, void* a, void* Cupd) {
-    if (h->prec == CH_F64) return launch_solve<double>(h, l, dir, (double*)a, (double*)Cupd, nullptr);
-    return launch_solve<float>(h, l, dir, (float*)a, (float*)Cupd, nullptr);
+int launch_solve_any(ch_handle* h, int l, int dir, const void* src, void* dst, void* Cupd) {
+    if (h->prec == CH_F64)
+        return launch_solve<double>(h, l, dir, (const double*)src, (double*)dst, (double*)Cupd, nullptr);
+    return launch_solve<float>(h, l, dir, (const float*)src, (float*)dst, (float*)Cupd, nullptr);
 }
 
 int launch_step_any(ch_handle* h, void* C) {
