@@ -607,7 +607,7 @@ ch_march_x(const T* src, T* dst, int64_t nlines, MarchCoef<T> k) {
 // ---------------------------------------------------------------------------
 // Most warps of a CTA: what leaves a thread room for its R rows (and R of C).
 template <int R>
-constexpr int tile_max_warps() { return R <= 16 ? 20 : 16; }
+constexpr int tile_max_warps() { return R <= 16 ? 20 : R <= 32 ? 16 : 8; }
 template <int R>
 __host__ __device__ constexpr int tile_warps(int n, int reach) { return (n + reach + R - 1) / R; }
 template <typename T, int R>

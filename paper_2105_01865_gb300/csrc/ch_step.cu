@@ -15,6 +15,7 @@
 
 #include "ch_internal.h"
 #include "ch_explicit2.cuh"
+#include "ch_explicit64.cuh"
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
 #include "ch_march.cuh"
@@ -547,17 +548,20 @@ bool multi_line_any(const ch_handle* h, int l, int dir) {
 //         500^3            old  311  356  390                         march  177  170  343
 //         1024 x 1024 x 512  old 1280 1420 1390                       march  663  648 1060
 //         1000 x 100 x 60, x only: old 26.4, march 36.9 (188 warps of 1000 rows)
-//   FP64  128^3            old  140  111  121  tile32   73   76   86  march  104  113  136
-//         256 x 256 x 128  old  382  444  369  tile32  218  217  266  march  258  281  359
+//   FP64  64^3             old   35   25   25  tile32   22   23   26  tile64   29   31   37
+//         128^3            old  140  111  121  tile32   73   76   86  tile64   62   68   77  march 104 113 136
+//         256 x 256 x 128  old  382  444  369  tile32  218  217  266  tile64  201  222  252  march 258 281 359
+//         200^3            old  465  629  587  tile32  203  229  254  tile64  176  198  227
 // So: the scan solvers where the operator decays too slowly, the restart is
 // longer than the line, or the line is short (whole steps with u = 0: FP32 64^3
 // old 59 us, new 70; 80^3 84 and 78; 128^3 113 and 92; FP64 64^3 471 and 436).  FP64, bound by its arithmetic, takes the form with the fewest
-// restarts, 32 rows a warp, where the line fits.  FP32 streams (march) once
+// restarts that still leaves every SM some warps: 64 rows a warp from 3
+// 32-line groups an SM on, else 32, where the line fits.  FP32 streams (march) once
 // 32-line groups outnumber the SMs two to one; fewer take 16 rows a warp, to
 // have warps enough; lines without 16-byte alignment, whose copies cost the
 // streaming warp an instruction an element, take 32 rows a warp up to 8 groups
 // an SM.  Long lines in few groups stay with the scans.
-enum LineForm { kLineScan, kLineTile16, kLineTile32, kLineMarch };
+enum LineForm { kLineScan, kLineTile16, kLineTile32, kLineTile64, kLineMarch };
 template <typename T>
 LineForm line_form(const ch_handle* h, int l, int dir) {
     const LineTables& lt = h->lines[dir][l];
@@ -565,10 +569,17 @@ LineForm line_form(const ch_handle* h, int l, int dir) {
     if (!lt.reach || lt.n < (sizeof(T) == 4 ? 65 : 64) || lt.reach > lt.n) return kLineScan;
     const int64_t groups = dir == 0 ? (ny * nz + 31) / 32 : dir == 1 ? (nx + 31) / 32 * nz : (nx * ny + 31) / 32;
     const int64_t row = dir == 2 ? nx * ny : nx;
-    const bool fits32 = tile_warps<32>(lt.n, lt.reach) <= tile_max_warps<32>() &&
-                        std::max(tile_yz_bytes<T, 32>(tile_warps<32>(lt.n, lt.reach)),
-                                 tile_x_bytes<T, 32>(tile_warps<32>(lt.n, lt.reach))) <= kMaxSmem;
-    if (sizeof(T) == 8) return fits32 ? kLineTile32 : groups >= 2 * 152 ? kLineMarch : kLineScan;
+    auto fits = [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int warps = tile_warps<R>(lt.n, lt.reach);
+        return warps <= tile_max_warps<R>() &&
+               std::max(tile_yz_bytes<T, R>(warps), tile_x_bytes<T, R>(warps)) <= kMaxSmem;
+    };
+    const bool fits32 = fits(std::integral_constant<int, 32>{});
+    if (sizeof(T) == 8) {
+        if (groups >= 3 * 152 && fits(std::integral_constant<int, 64>{})) return kLineTile64;
+        return fits32 ? kLineTile32 : groups >= 2 * 152 ? kLineMarch : kLineScan;
+    }
     if (row % 4 != 0 && fits32 && groups <= 8 * 152) return kLineTile32;
     if (groups <= 2 * 152 && tile_warps<16>(lt.n, lt.reach) <= tile_max_warps<16>()) return kLineTile16;
     return groups >= 2 * 152 ? kLineMarch : kLineScan;
@@ -688,6 +699,8 @@ int set_attrs_march(ch_handle* h) {
     }
     if constexpr (sizeof(T) == 4)
         if (rc == CH_OK) rc = set_attrs_tile<T, 16>(h);
+    if constexpr (sizeof(T) == 8)
+        if (rc == CH_OK) rc = set_attrs_tile<T, 64>(h);
     if (rc == CH_OK) rc = set_attrs_tile<T, 32>(h);
     return rc;
 }
@@ -698,6 +711,9 @@ int launch_solve(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd, cuda
     switch (line_form<T>(h, l, dir)) {
         case kLineMarch: rc = launch_march<T>(h, l, dir, src, r, Cupd); break;
         case kLineTile32: rc = launch_tile<T, 32>(h, l, dir, src, r, Cupd); break;
+        case kLineTile64:
+            if constexpr (sizeof(T) == 8) rc = launch_tile<T, 64>(h, l, dir, src, r, Cupd);
+            break;
         case kLineTile16:
             if constexpr (sizeof(T) == 4) rc = launch_tile<T, 16>(h, l, dir, src, r, Cupd);
             break;
@@ -793,7 +809,29 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
     const T* v = p.advect ? (const T*)h->vel[1] : nullptr;
     const T* w = p.advect ? (const T*)h->vel[2] : nullptr;
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[0], h->stream));
-    if (nx % 2 == 0) {  // two cells per thread (paired FP32 arithmetic)
+    if constexpr (sizeof(T) == 8) {
+        const bool diri = p.bc[2] == CH_DIRICHLET;
+        // 8-row tiles, 3 CTAs an SM: 2757 us on the 256 x 256 x 128 shear drop,
+        // 2835 with 2 CTAs, 2913 with 16-row tiles (1 CTA: every warp meets at
+        // the same barriers).  A z-chunk costs about half a plane to start:
+        // 16 planes, halved while that leaves fewer than 6 CTAs an SM (64^3: 91
+        // us with 56 CTAs of 10 planes, 35 with 512 of 2).
+        constexpr int TY = 8, MINB = 3;
+        const int64_t xy = (int64_t)((nx + kEX - 1) / kEX) * ((ny + TY - 1) / TY);
+        int tz = 16;
+        while (tz > 2 && xy * ((nz + tz - 1) / tz) < 6 * 152) tz /= 2;
+        const dim3 grid((nx + kEX - 1) / kEX, (ny + TY - 1) / TY, (nz + tz - 1) / tz), block(kEX, TY);
+        auto go = [&](auto adv, auto dir) {
+            launch_k(h->stream, ch_explicit_f64<decltype(adv)::value, decltype(dir)::value, TY, MINB>, grid, block, 0, C, u,
+                     v, w, Hprev, Hout, r, a, tz);
+        };
+        using Yes = std::true_type;
+        using No = std::false_type;
+        if (p.advect && diri) go(Yes{}, Yes{});
+        else if (p.advect) go(Yes{}, No{});
+        else if (diri) go(No{}, Yes{});
+        else go(No{}, No{});
+    } else if (nx % 2 == 0) {  // two cells per thread (paired FP32 arithmetic)
         const int tz = explicit_zchunk(nx, ny, nz, sizeof(T) == 4);
         dim3 grid((nx + kTX2 - 1) / kTX2, (ny + kTY - 1) / kTY, (nz + tz - 1) / tz);
         dim3 block(32, kTY);
@@ -823,17 +861,13 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
                          Hout, r, a, tm, h->status);
         };
         using NoTma = std::false_type;
-        if constexpr (sizeof(T) == 4) {
-            using Tma = std::integral_constant<bool, CH_EXPLICIT_TMA != 0>;
-            if (tz == kTZ2Deep) {
-                if (tma) go(std::integral_constant<int, kTZ2Deep>{}, Tma{});
-                else go(std::integral_constant<int, kTZ2Deep>{}, NoTma{});
-            } else {
-                if (tma) go(std::integral_constant<int, kTZ2>{}, Tma{});
-                else go(std::integral_constant<int, kTZ2>{}, NoTma{});
-            }
+        using Tma = std::integral_constant<bool, CH_EXPLICIT_TMA != 0>;
+        if (tz == kTZ2Deep) {
+            if (tma) go(std::integral_constant<int, kTZ2Deep>{}, Tma{});
+            else go(std::integral_constant<int, kTZ2Deep>{}, NoTma{});
         } else {
-            go(std::integral_constant<int, kTZ2>{}, NoTma{});
+            if (tma) go(std::integral_constant<int, kTZ2>{}, Tma{});
+            else go(std::integral_constant<int, kTZ2>{}, NoTma{});
         }
     } else {
         dim3 grid((nx + kTX - 1) / kTX, (ny + kTY - 1) / kTY, (nz + kTZ - 1) / kTZ);
