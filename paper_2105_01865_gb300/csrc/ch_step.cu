@@ -14,7 +14,7 @@
 #include <vector>
 
 #include "ch_internal.h"
-#include "ch_explicit2.cuh"
+#include "ch_explicit3.cuh"
 #include "ch_explicit64.cuh"
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
@@ -88,19 +88,11 @@ constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory per CTA (sm_10
 #ifndef CH_YZ_PERSIST
 #define CH_YZ_PERSIST 0
 #endif
-// shortest lines (in rows per lane, M) that take the multi-line solvers
-// FP32 explicit kernel: stage C through a tensor map (TMA tile loads, two
-// planes ahead) on the tiles that need no wrapped or mirrored index.  Off by
-// default: measured slower than the per-thread copies on the 1024x1024x512
-// mesh (5.67 against 5.58 ms per launch; the kernel is bound by instruction
-// issue, not by its staging)
-#ifndef CH_EXPLICIT_TMA
-#define CH_EXPLICIT_TMA 0
-#endif
 // CTAs per SM of the mass and free-energy reductions
 #ifndef CH_RED_BLOCKS_PER_SM
 #define CH_RED_BLOCKS_PER_SM 4
 #endif
+// shortest lines (in rows per lane, M) that take the multi-line solvers
 #ifndef CH_MULTI_MIN_M
 #define CH_MULTI_MIN_M 16
 #endif
@@ -771,6 +763,27 @@ int set_attrs_m(ch_handle* h) {
 // Explicit RHS of substep l from C (and Hprev) into Hout and r.
 // With adv_only (the standard scheme's advection): Hout = -div(uC) only, no
 // diffusive or implicit term, no right-hand side written.
+// Planes a tile marches: the depth whose waves of CTAs take the least, a tile
+// costing its planes and about kTileStart more (its z-queue and first copies).
+// Against fixed depths: 256 x 256 x 128, 91 us (19 planes) and 92 (16) or 114
+// (64); 500^3, 1211 us (56) and 1333 (64); 64^3 without advection, 7 us (2)
+// and 11 (10); 1024 x 1024 x 512, 4.85 ms either way (64).
+inline int explicit_depth(int64_t xy, int nz, int64_t slots) {
+    constexpr double kTileStart = 2.0;
+    int best = nz;
+    double least = 0.0;
+    for (int c = 1; c <= nz; ++c) {
+        const int tz = (nz + c - 1) / c;
+        const int64_t ctas = xy * ((nz + tz - 1) / tz);
+        const double cost = (double)((ctas + slots - 1) / slots) * (tz + kTileStart);
+        if (c == 1 || cost < least) {
+            least = cost;
+            best = tz;
+        }
+    }
+    return best;
+}
+
 template <typename T>
 int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T* r, cudaEvent_t* ev,
                     bool adv_only = false) {
@@ -831,51 +844,28 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
         else if (p.advect) go(Yes{}, No{});
         else if (diri) go(No{}, Yes{});
         else go(No{}, No{});
-    } else if (nx % 2 == 0) {  // two cells per thread (paired FP32 arithmetic)
-        const int tz = explicit_zchunk(nx, ny, nz, sizeof(T) == 4);
-        dim3 grid((nx + kTX2 - 1) / kTX2, (ny + kTY - 1) / kTY, (nz + tz - 1) / tz);
-        dim3 block(32, kTY);
-        const bool diri = p.bc[2] == CH_DIRICHLET;
-        // the tensor map of the handle's C (FP32) when this launch reads that C
-        CUtensorMap tm;
-        std::memcpy(&tm, h->tmap_c, sizeof(tm));
-        // ... and when most tiles (>= 3/4) need no wrapped or mirrored index, so
-        // take the tile load; the rest stage element by element
-        const int64_t txn = (nx + kTX2 - 1) / kTX2, tyn = (ny + kTY - 1) / kTY;
-        const bool mostly_inner = 4 * std::max<int64_t>(txn - 2, 0) * std::max<int64_t>(tyn - 2, 0) >= 3 * txn * tyn;
-        const bool tma = sizeof(T) == 4 && h->tmap_ok && (const void*)C == h->C && mostly_inner;
-        auto go = [&](auto tzc, auto tmac) {
-            constexpr int TZ = decltype(tzc)::value;
-            constexpr bool TMA = decltype(tmac)::value;
-            if (p.advect && diri)
-                launch_k(h->stream, ch_explicit_rhs2<T, true, true, TZ, TMA>, grid, block, 0, C, u, v, w, Hprev, Hout,
-                         r, a, tm, h->status);
-            else if (p.advect)
-                launch_k(h->stream, ch_explicit_rhs2<T, true, false, TZ, TMA>, grid, block, 0, C, u, v, w, Hprev, Hout,
-                         r, a, tm, h->status);
-            else if (diri)
-                launch_k(h->stream, ch_explicit_rhs2<T, false, true, TZ, TMA>, grid, block, 0, C, u, v, w, Hprev, Hout,
-                         r, a, tm, h->status);
-            else
-                launch_k(h->stream, ch_explicit_rhs2<T, false, false, TZ, TMA>, grid, block, 0, C, u, v, w, Hprev,
-                         Hout, r, a, tm, h->status);
-        };
-        using NoTma = std::false_type;
-        using Tma = std::integral_constant<bool, CH_EXPLICIT_TMA != 0>;
-        if (tz == kTZ2Deep) {
-            if (tma) go(std::integral_constant<int, kTZ2Deep>{}, Tma{});
-            else go(std::integral_constant<int, kTZ2Deep>{}, NoTma{});
-        } else {
-            if (tma) go(std::integral_constant<int, kTZ2>{}, Tma{});
-            else go(std::integral_constant<int, kTZ2>{}, NoTma{});
-        }
     } else {
-        dim3 grid((nx + kTX - 1) / kTX, (ny + kTY - 1) / kTY, (nz + kTZ - 1) / kTZ);
-        dim3 block(kTX, kTY);
-        if (p.advect)
-            launch_k(h->stream, ch_explicit_rhs<T, true>, dim3(grid), dim3(block), 0, C, u, v, w, Hprev, Hout, r, a);
-        else
-            launch_k(h->stream, ch_explicit_rhs<T, false>, dim3(grid), dim3(block), 0, C, u, v, w, Hprev, Hout, r, a);
+        const bool diri = p.bc[2] == CH_DIRICHLET;
+        const int64_t xy = (int64_t)((nx + kTX2 - 1) / kTX2) * ((ny + kTY - 1) / kTY);
+        const int xm = nx % 4 ? kRowsAny : p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsWalled;
+        const int tz = explicit_depth(xy, nz, 152 * (xm == kRowsAny ? 2 : 3));
+        const dim3 grid((nx + kTX2 - 1) / kTX2, (ny + kTY - 1) / kTY, (nz + tz - 1) / tz), block(32, kTY);
+        auto go = [&](auto adv, auto dir, auto xmc) {
+            // without H^{l-1} its copies have length 0: any valid source
+            launch_k(h->stream, ch_explicit_rhs3<decltype(adv)::value, decltype(dir)::value, decltype(xmc)::value>, grid,
+                     block, 0, C, u, v, w, Hprev ? Hprev : C, Hout, r, a, tz);
+        };
+        using Yes = std::true_type;
+        using No = std::false_type;
+        auto go2 = [&](auto xmc) {
+            if (p.advect && diri) go(Yes{}, Yes{}, xmc);
+            else if (p.advect) go(Yes{}, No{}, xmc);
+            else if (diri) go(No{}, Yes{}, xmc);
+            else go(No{}, No{}, xmc);
+        };
+        if (xm == kRowsPeriodic) go2(std::integral_constant<int, kRowsPeriodic>{});
+        else if (xm == kRowsWalled) go2(std::integral_constant<int, kRowsWalled>{});
+        else go2(std::integral_constant<int, kRowsAny>{});
     }
     CHG_CUDA(h, cudaGetLastError());
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[1], h->stream));
@@ -1012,38 +1002,6 @@ size_t ch_workspace_bytes(const ch_params* p) {
     return layout(p).total;
 }
 
-// The explicit kernel's tensor map of C: FP32, nx a multiple of 4 (16-byte
-// row strides), a box of one staged plane (72 x 14 x 1).  Left unset
-// (tmap_ok = 0) when the driver entry point or the encoding is unavailable;
-// the kernel then stages every tile element by element.
-void encode_tmap_c(ch_handle* h) {
-    h->tmap_ok = 0;
-    if (!CH_EXPLICIT_TMA || h->prec != CH_F32 || h->n[0] % 4 != 0) return;
-    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-            cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn) {
-        cudaGetLastError();
-        return;
-    }
-    const cuuint64_t dims[3] = {(cuuint64_t)h->n[0], (cuuint64_t)h->n[1], (cuuint64_t)h->n[2]};
-    const cuuint64_t strides[2] = {(cuuint64_t)h->n[0] * 4, (cuuint64_t)(h->n[0] * h->n[1]) * 4};
-    const cuuint32_t box[3] = {(cuuint32_t)(kTX2 + 2 * kHL2), (cuuint32_t)(kTY + 2 * kHalo), 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUtensorMap tm;
-    if (((Encode)fn)(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->C, dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return;
-    static_assert(sizeof(tm) == sizeof(h->tmap_c), "tensor map size");
-    std::memcpy(h->tmap_c, &tm, sizeof(tm));
-    h->tmap_ok = 1;
-}
-
 int ch_create(const ch_params* p, void* C, void* work, size_t work_bytes, void* stream, ch_handle** out) {
     char why[256];
     if (!out) return CH_EINVAL;
@@ -1174,7 +1132,6 @@ int ch_create(const ch_params* p, void* C, void* work, size_t work_bytes, void* 
             rc = CH_ECUDA;
     }
     if (rc == CH_OK) rc = h->prec == CH_F64 ? set_smem_attrs<double>(h) : set_smem_attrs<float>(h);
-    if (rc == CH_OK) encode_tmap_c(h);
     if (rc == CH_OK && p->ncx) rc = mr_build_tables(h, p->xf_coarse, p->yf_coarse, p->zf_coarse);
     if (rc == CH_OK && p->ncx) rc = rs_build_tables(h, p->xf_coarse, p->yf_coarse, p->zf_coarse);
     if (rc != CH_OK) {
@@ -1283,7 +1240,6 @@ int ch_sync(ch_handle* h) {
     if (flag) {
         CHG_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(unsigned int), h->stream));
         CHG_CUDA(h, cudaStreamSynchronize(h->stream));
-        if (flag & 4u) return fail(h, CH_ETIMEOUT, "a tile load of the explicit kernel did not complete");
         return fail(h, CH_ENONFINITE, "non-finite value in C");
     }
     return CH_OK;

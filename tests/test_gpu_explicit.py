@@ -1,5 +1,5 @@
-"""GPU tests of the FP64 explicit kernel at the edges of its 32-wide tiles and
-of its z-chunks: two steps with a flow that changes sign, against the oracle."""
+"""GPU tests of the explicit kernels at the edges of their tiles, copies and
+z-chunks: two steps with a flow that changes sign, against the oracle."""
 import numpy as np
 import pytest
 
@@ -48,3 +48,30 @@ def test_two_steps_match_oracle(shape, bc, flow):
     ref = co.step(C0, vel, p, 2)
     # the bar of the other FP64 tests; rounding alone gives about 1e-15
     assert_parity(got, ref, 1e-12, f"FP64 explicit {shape} {bc} flow={flow}")
+
+
+# the FP32 kernel's copies: whole 16-byte chunks (nx a multiple of 4; walls
+# reverse the last one), element by element otherwise, a lone last column
+@pytest.mark.parametrize("nx", [5, 8, 12, 63, 64, 65, 66, 68, 129])
+@pytest.mark.parametrize("bc", [(P, P, P), (N, P, N), (N, N, D)])
+@pytest.mark.parametrize("flow", [True, False])
+def test_fp32_two_steps_match_oracle(nx, bc, flow):
+    from paper_2105_01865_gb300.solver import Solver
+    nz, ny = 9, 17
+    shape = (nz, ny, nx)
+    h, cn, pe = 1.0 / 16, 0.75 / 16, 20.0
+    rng = np.random.default_rng(nx)
+    C0 = (0.5 + 0.4 * rng.standard_normal(shape)).astype(np.float32).astype(np.float64)
+    vel = None
+    if flow:
+        vel = inputs.curl_velocity(*(inputs.uniform_faces(n, n * h) for n in (nx, ny, nz)), bc, seed=nx, kmax=3)
+        vel = [a.astype(np.float32).astype(np.float64) for a in vel]
+    s = Solver(shape, h, bc, cn, pe, 0.2 * h, C0, precision="f32", advect=flow)
+    if flow:
+        s.set_velocity_fine(*vel)
+    s.step(2)
+    got = s.field()
+    s.close()
+    ref = co.step(C0, vel, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=0.2 * h, bc=bc), 2)
+    # the bar of the other FP32 tests of a few steps
+    assert_parity(got, ref, 1e-6, f"FP32 explicit {shape} {bc} flow={flow}")
