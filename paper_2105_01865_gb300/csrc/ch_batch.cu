@@ -27,6 +27,7 @@
 #include "ch_explicit2.cuh"
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
+#include "ch_explicit3.cuh"
 #include "line_tables.h"
 
 using namespace chg;
@@ -50,6 +51,7 @@ struct BoxDesc {
     // 0 where the line is too long and the shared-memory tile solver runs
     int colR[2];
     CCoef<float> cols[2][kRK];
+    int rows;  // kRowsAny, kRowsWalled or kRowsPeriodic
 };
 
 struct BatchArgs {
@@ -157,8 +159,14 @@ __device__ void run_phase(const BatchArgs& A, int ph, int l, float* smem) {
         const int4 w = items[it];
         const BoxDesc& B = A.boxes[w.x];
         if (ph == 0) {
-            explicit_tile2<float, false>(B.C, nullptr, nullptr, nullptr, B.H[(l + 1) & 1], B.H[l & 1], B.r, B.rhs[l],
-                                         w.y, w.z, w.w, A.zchunk);
+            Explicit3Smem<false>& sm = *reinterpret_cast<Explicit3Smem<false>*>(smem);
+            float *Hp = B.H[(l + 1) & 1], *Ho = B.H[l & 1];
+            if (B.rows == kRowsPeriodic)
+                explicit_tile3<false, false, kRowsPeriodic>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z,
+                                                            w.w, A.zchunk, sm);
+            else
+                explicit_tile3<false, false, kRowsAny>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z, w.w,
+                                                       A.zchunk, sm);
         } else if (ph == 1) {
             switch (B.M[0]) {
                 case 1: x_item<1>(B, w.y, l); break;
@@ -287,7 +295,7 @@ struct ch_batch {
     int red_blocks = 64;
     // schedule
     int mode = 0;  // 0 persistent, 1 phased
-    int blocks_per_sm = 2;
+    int blocks_per_sm = 3;  // 2.64 ms a step against 3.44 with 2 on the 64 uneven boxes of the bench (57.6 M cells)
     int zchunk = 8;
     int lpt = 1;
     long long limit_ns = 2000000000LL;
@@ -490,6 +498,7 @@ int ch_batch_create(const ch_params* boxes, int nbox, void* const* C, void* work
         B.ny = (int)p.ny;
         B.nz = (int)p.nz;
         B.nlines_x = (int)(p.ny * p.nz);
+        B.rows = p.nx % 4 == 0 && p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsAny;
         const double mob = 1.0 / p.pe;
         const double kappa = p.w * p.cn * p.cn / (p.h * p.h * p.h * p.h);
         for (int l = 0; l < kRK; ++l) {
@@ -534,7 +543,7 @@ int ch_batch_create(const ch_params* boxes, int nbox, void* const* C, void* work
         }
     }
     // dynamic shared memory: the larger of the y/z tile and the two-column buffers
-    b->smem = (size_t)32 * maxM * 32 * sizeof(float);
+    b->smem = std::max(sizeof(Explicit3Smem<false>), (size_t)32 * maxM * 32 * sizeof(float));
     if (maxR) b->smem = std::max(b->smem, cols2_smem_max(maxR));
     b->max_m = maxM;
     int rc = CH_OK;
