@@ -229,10 +229,6 @@ struct BlockSum {
 // reads per ix per CTA.  Otherwise each warp contracts its 16 rows itself.
 constexpr int kMrWarps = 8;
 constexpr int kMrQRows = 8;
-// adjacent fine columns per thread of the y/z line march (1, 2 or 4)
-#ifndef CH_MR_CPT
-#define CH_MR_CPT 4
-#endif
 constexpr size_t kMrMaxSmem = 226 * 1024;  // dynamic shared memory per CTA (227 KB on sm_103a, less the static)
 
 template <typename T>
@@ -475,8 +471,9 @@ struct MrVec<double, 2> {
     }
 };
 
+constexpr int kLineThreads = 64;
 template <typename T, int DIR, int CPT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kLineThreads)
 mr_line_yz(const T* __restrict__ P, const T* __restrict__ Vc, Tab<T> tx, Tab<T> ty, Tab<T> tz, MrArgs a,
            T* __restrict__ out) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -612,17 +609,25 @@ int interp(ch_handle* h, cudaEvent_t* ev = nullptr) {
     }
     T* P = (T*)h->mr_plane;
     const size_t zsm = (size_t)a.ncx * sizeof(T);
-    // the line march with CPT adjacent columns per thread where nx allows
-    constexpr int CPT = sizeof(T) == 4 ? CH_MR_CPT : (CH_MR_CPT < 2 ? CH_MR_CPT : 2);
+    // The line march is one long chain a thread, so the threads have to fill the
+    // chip before columns are put together: CPT adjacent columns a thread while
+    // that leaves 700 threads an SM, in CTAs of 64 threads so that they spread.
+    // 512 x 512 x 256: y 166 -> 158 us with 1 column instead of 4 (128 CTAs of 256
+    // threads left SMs idle), z 104 -> 95 with 2; 1024 x 1024 x 512 keeps 4 (y 874
+    // us, with 2 1062).
+    constexpr int kMost = sizeof(T) == 4 ? 4 : 2;
     auto line = [&](auto dirc, const T* Vc, T* out, int64_t ntr) {
         constexpr int DIR = decltype(dirc)::value;
-        if (a.nx % CPT == 0) {
+        auto go = [&](auto cptc) {
+            constexpr int CPT = decltype(cptc)::value;
             const int64_t thr = (int64_t)(a.nx / CPT) * ntr;
-            mr_line_yz<T, DIR, CPT><<<(unsigned)((thr + 255) / 256), 256, 0, h->stream>>>(P, Vc, tx, ty, tz, a, out);
-        } else {
-            const int64_t thr = (int64_t)a.nx * ntr;
-            mr_line_yz<T, DIR, 1><<<(unsigned)((thr + 255) / 256), 256, 0, h->stream>>>(P, Vc, tx, ty, tz, a, out);
-        }
+            mr_line_yz<T, DIR, CPT><<<(unsigned)((thr + kLineThreads - 1) / kLineThreads), kLineThreads, 0, h->stream>>>(
+                P, Vc, tx, ty, tz, a, out);
+        };
+        auto fits = [&](int cpt) { return a.nx % cpt == 0 && (int64_t)(a.nx / cpt) * ntr >= 700 * 152; };
+        if (kMost == 4 && fits(4)) go(std::integral_constant<int, kMost>{});
+        else if (fits(2)) go(std::integral_constant<int, 2>{});
+        else go(std::integral_constant<int, 1>{});
     };
     {
         mr_plane_yz<T, 1><<<16 * 152, 256, zsm, h->stream>>>((const T*)h->grad_c[1], tx, ty, tz, a, P);
