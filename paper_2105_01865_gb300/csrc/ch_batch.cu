@@ -24,7 +24,7 @@
 #include <vector>
 
 #include "ch_internal.h"
-#include "ch_explicit2.cuh"
+#include "ch_pairs.cuh"
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
 #include "ch_explicit3.cuh"

@@ -16,7 +16,7 @@
 
 #include <cooperative_groups.h>
 
-#include "ch_explicit2.cuh"
+#include "ch_pairs.cuh"
 
 namespace chg {
 
@@ -36,10 +36,6 @@ struct Cols2Smem {
 __device__ __forceinline__ void cp_async_pair(Pr<float>* dst, const float* src) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_pair(Pr<double>* dst, const double* src) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(src) : "memory");
 }
 
 // Coefficient loads: volatile (issued in program order, so the compiler

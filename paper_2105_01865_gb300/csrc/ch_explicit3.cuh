@@ -28,7 +28,7 @@
 // go element by element.
 #pragma once
 
-#include "ch_explicit2.cuh"
+#include "ch_pairs.cuh"
 
 namespace chg {
 

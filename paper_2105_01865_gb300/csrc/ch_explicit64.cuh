@@ -15,8 +15,8 @@
 // for a negative velocity, F the same function, so the sign only turns the
 // direction in which the shared line is read.
 //
-// 256 x 256 x 128 shear drop, with advection: 3641 us a launch with the paired
-// kernel of ch_explicit2.cuh, 2586 with this one, about 160 FP64 operations a
+// 256 x 256 x 128 shear drop, with advection: 3641 us a launch when
+// it shared the paired FP32 design, 2586 so, about 160 FP64 operations a
 // cell at 85 % of the FP64 pipe.  64^3 without: 91 and 35 us.
 #pragma once
 

@@ -1,9 +1,8 @@
 // Device kernels of the Cahn-Hilliard fine-grid step (arXiv 2105.01865, Sec. 3).
 //
-//  ch_explicit_rhs   explicit terms of one RK3 substep + right-hand side of
-//                    the delta-form Crank-Nicolson system (Eq. eq-re):
-//                    H^l = -div(u C) + M lap(psi'(C)),
-//                    r   = dt (gamma_l H^l + rho_l H^{l-1}) - alpha_l dt M sum_d A_d C
+//  (ch_explicit3.cuh, ch_explicit64.cuh: the explicit terms of a substep and the
+//   right-hand side of the delta-form Crank-Nicolson system, Eq. eq-re;
+//   ch_march.cuh: the line solves of operators that decay along the line)
 //  ch_solve_x        (I + (alpha_l dt M / 2) A_x) dq*  = r     (Eq. eq-fac-1)
 //  ch_solve_yz       (I + (alpha_l dt M / 2) A_y) dq** = dq*   (Eq. eq-fac-2)
 //                    (I + (alpha_l dt M / 2) A_z) dq   = dq**, C += dq (Eq. eq-fac-3)
@@ -21,9 +20,7 @@
 
 namespace chg {
 
-constexpr int kTX = 32;   // explicit-kernel tile, x (one warp)
 constexpr int kTY = 8;    // explicit-kernel tile, y (warps per CTA)
-constexpr int kTZ = 16;   // z-planes marched per CTA
 constexpr int kHalo = 3;  // WENO5 needs three cells on each side
 
 template <typename T>
@@ -68,43 +65,6 @@ __device__ __forceinline__ int bc_near(int i, int n, int bc) {
     return i;
 }
 
-template <typename T>
-__device__ __forceinline__ T psi_p(T c) {  // psi'(C) = C^3 - 1.5 C^2 + 0.5 C (Eq. eq-ch)
-    return c * (c * (c - T(1.5)) + T(0.5));
-}
-
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
-
-// Fifth-order WENO (Jiang-Shu) value at the face between v3 and v4 from the
-// upwind-biased stencil v1..v5 (Sec. 3: "fifth-order WENO").  The nonlinear
-// weights alpha_k = d_k / (eps + beta_k)^2, normalised, are formed over a
-// common denominator so that one division serves all three.
-template <typename T>
-__device__ __forceinline__ T weno5(T v1, T v2, T v3, T v4, T v5, T eps) {
-    const T q0 = T(2) * v1 - T(7) * v2 + T(11) * v3;   // 6 x candidate values
-    const T q1 = -v2 + T(5) * v3 + T(2) * v4;
-    const T q2 = T(2) * v3 + T(5) * v4 - v5;
-    const T d0 = v1 - T(2) * v2 + v3, e0 = v1 - T(4) * v2 + T(3) * v3;
-    const T d1 = v2 - T(2) * v3 + v4, e1 = v2 - v4;
-    const T d2 = v3 - T(2) * v4 + v5, e2 = T(3) * v3 - T(4) * v4 + v5;
-    const T s0 = eps + (T(13.0 / 12.0) * d0 * d0 + T(0.25) * e0 * e0);
-    const T s1 = eps + (T(13.0 / 12.0) * d1 * d1 + T(0.25) * e1 * e1);
-    const T s2 = eps + (T(13.0 / 12.0) * d2 * d2 + T(0.25) * e2 * e2);
-    const T t0 = s0 * s0, t1 = s1 * s1, t2 = s2 * s2;
-    const T w0 = T(0.1) * (t1 * t2), w1 = T(0.6) * (t0 * t2), w2 = T(0.3) * (t0 * t1);
-    return fdiv(w0 * q0 + w1 * q1 + w2 * q2, T(6) * (w0 + w1 + w2));
-}
-
-// Flux u_f C_f through a face, C_f from the upwind WENO5 stencil.  m3..p2 are
-// the cells f-3 .. f+2 around the face f (between cells f-1 and f).
-template <typename T>
-__device__ __forceinline__ T face_flux(T vel, T m3, T m2, T m1, T p0, T p1, T p2, T eps) {
-    const bool up = vel >= T(0);
-    const T a1 = up ? m3 : p2, a2 = up ? m2 : p1, a3 = up ? m1 : p0, a4 = up ? p0 : m1, a5 = up ? p1 : m2;
-    return vel * weno5(a1, a2, a3, a4, a5, eps);
-}
-
 // Programmatic dependent launch.  A kernel launched with programmatic stream
 // serialisation may be scheduled while its predecessor drains; pdl_wait()
 // blocks until the predecessor grid has completed and its writes are
@@ -135,244 +95,9 @@ __device__ __forceinline__ void cp_async_16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
-// Tensor-memory-accelerator (TMA) tile loads completed on a shared-memory
-// mbarrier (transaction count in bytes).
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-// make barrier initialisation visible to the async proxy (the TMA unit)
-__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-    return t;
-}
-// Wait for phase `parity` of the barrier, giving up after `limit_ns`.
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity, unsigned long long limit_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(bar, parity))
-        if (global_ns() - t0 > limit_ns) return false;
-    return true;
-}
-// 3D tile (x innermost) of a tensor map into shared memory; x must be a
-// multiple of 16 bytes of elements, the destination 128-byte aligned.
-__device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, int x, int y, int z, unsigned long long* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];\n" ::"r"(smem_u32(dst)),
-        "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-        : "memory");
-}
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-// ---------------------------------------------------------------------------
-// Explicit right-hand side.  A CTA owns a 32 x 8 column of cells and marches
-// kTZ planes in z.  Each plane (with a 3-cell halo in x and y) is staged in
-// shared memory through per-CTA index tables (no division in the loop); the
-// cell's own z-column lives in a 6-register queue.  Every face flux is
-// computed exactly once (lower faces by their cell, the extra upper faces of
-// the tile by dedicated lanes, z-faces carried between planes), so the
-// fluxes telescope bit-exactly and mass is conserved to rounding.
-// ---------------------------------------------------------------------------
-template <typename T, bool ADV>
-__global__ void __launch_bounds__(kTX * kTY)
-ch_explicit_rhs(const T* __restrict__ C, const T* __restrict__ u, const T* __restrict__ v,
-                const T* __restrict__ w, const T* __restrict__ Hprev, T* __restrict__ Hout,
-                T* __restrict__ r, RhsArgs<T> a) {
-    pdl_wait();
-    pdl_launch_dependents();
-    constexpr int PX = kTX + 2 * kHalo, PY = kTY + 2 * kHalo;
-    __shared__ __align__(16) T Cs[3][PY][PX];
-    __shared__ T Fx[ADV ? kTY : 1][kTX + 1];
-    __shared__ T Fy[ADV ? kTY + 1 : 1][kTX];
-    __shared__ int gi_tab[PX], gj_tab[PY];
-
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kTX + tx;
-    const int i0 = blockIdx.x * kTX, j0 = blockIdx.y * kTY, k0 = blockIdx.z * kTZ;
-    const int i = i0 + tx, j = j0 + ty;
-    const bool in_xy = (i < a.nx) && (j < a.ny);
-    const int ic = min(i, a.nx - 1), jc = min(j, a.ny - 1);
-    const int64_t plane = (int64_t)a.nx * a.ny;
-    const int64_t col = (int64_t)jc * a.nx + ic;
-    const T eps = a.eps;
-    const int kend = min(k0 + kTZ, a.nz);
-
-    if (tid < PX) gi_tab[tid] = bc_index(i0 + tid - kHalo, a.nx, a.bcx);
-    else if (tid < PX + PY) gj_tab[tid - PX] = bc_index(j0 + (tid - PX) - kHalo, a.ny, a.bcy);
-
-    // face indices and wall flags of this thread's faces (fixed over the march)
-    const bool wall_x = (a.bcx == CH_NOFLUX) && (i <= 0 || i >= a.nx);
-    const int fi = (a.bcx == CH_PERIODIC) ? bc_index(i, a.nx, CH_PERIODIC) : min(i, a.nx);
-    const bool wall_y = (a.bcy == CH_NOFLUX) && (j <= 0 || j >= a.ny);
-    const int fj = (a.bcy == CH_PERIODIC) ? bc_index(j, a.ny, CH_PERIODIC) : min(j, a.ny);
-    // extra faces: x-face i0+32 of row (j0 + tx) for warp 0 lanes < 8, y-face j0+8 for warp 1
-    const int ie = i0 + kTX, je_row = min(j0 + tx, a.ny - 1);
-    const bool wall_xe = (a.bcx == CH_NOFLUX) && (ie >= a.nx);
-    const int fie = (a.bcx == CH_PERIODIC) ? bc_index(ie, a.nx, CH_PERIODIC) : min(ie, a.nx);
-    const int je = j0 + kTY;
-    const bool wall_ye = (a.bcy == CH_NOFLUX) && (je >= a.ny);
-    const int fje = (a.bcy == CH_PERIODIC) ? bc_index(je, a.ny, CH_PERIODIC) : min(je, a.ny);
-
-    // z-column queue: q[m] = C(ic, jc, k - 2 + m), m = 0..5
-    T q[6];
-#pragma unroll
-    for (int m = 0; m < 6; ++m) {
-        q[m] = C[(int64_t)bc_near(k0 - 2 + m, a.nz, a.bcz) * plane + col];
-        if (bc_negate(k0 - 2 + m, a.nz, a.bcz)) q[m] = -q[m];
-    }
-
-    T fz_lo = T(0);
-    if (ADV) {
-        // flux through the lower z-face of plane k0
-        const bool wall = (a.bcz != CH_PERIODIC) && (k0 == 0);
-        if (!wall) {
-            T cm3 = C[(int64_t)bc_near(k0 - 3, a.nz, a.bcz) * plane + col];
-            if (bc_negate(k0 - 3, a.nz, a.bcz)) cm3 = -cm3;
-            const T wv = w[(int64_t)k0 * plane + col];
-            fz_lo = face_flux(wv, cm3, q[0], q[1], q[2], q[3], q[4], eps);
-        }
-    }
-    __syncthreads();  // index tables ready
-
-    // Planes are staged with asynchronous 4/8-byte copies into a ring of three
-    // buffers: plane k+1 is in flight while plane k is computed, and the
-    // buffer being refilled was last read two planes ago (behind a barrier).
-    auto stage = [&](int kk, int b) {
-        const T* Ck = C + (int64_t)kk * plane;
-        for (int e = tid; e < PX * PY; e += kTX * kTY) {
-            const int row = e / PX, cc = e - row * PX;
-            cp_async_elem(&Cs[b][row][cc], Ck + (int64_t)gj_tab[row] * a.nx + gi_tab[cc]);
-        }
-        cp_async_commit();
-    };
-    stage(k0, 0);
-    for (int k = k0, buf = 0; k < kend; ++k, buf = (buf == 2 ? 0 : buf + 1)) {
-        if (k + 1 < kend) {
-            stage(k + 1, buf == 2 ? 0 : buf + 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        // prefetch the next queue entry C(k + 4)
-        T qnext = C[(int64_t)bc_near(k + 4, a.nz, a.bcz) * plane + col];
-        if (bc_negate(k + 4, a.nz, a.bcz)) qnext = -qnext;
-        __syncthreads();
-
-        const int cy = ty + kHalo, cx = tx + kHalo;
-        T fz_up = T(0);
-        if (ADV) {
-            const int64_t kp = (int64_t)k * a.ny;
-            // x: flux through this cell's lower face (face i)
-            {
-                T f = T(0);
-                if (!wall_x) {
-                    const T uv = u[(kp + jc) * a.nfx + fi];
-                    f = face_flux(uv, Cs[buf][cy][cx - 3], Cs[buf][cy][cx - 2], Cs[buf][cy][cx - 1],
-                                  Cs[buf][cy][cx], Cs[buf][cy][cx + 1], Cs[buf][cy][cx + 2], eps);
-                }
-                Fx[ty][tx] = f;
-            }
-            // y: flux through this cell's lower face (face j)
-            {
-                T f = T(0);
-                if (!wall_y) {
-                    const T vv = v[((int64_t)k * a.nfy + fj) * a.nx + ic];
-                    f = face_flux(vv, Cs[buf][cy - 3][cx], Cs[buf][cy - 2][cx], Cs[buf][cy - 1][cx],
-                                  Cs[buf][cy][cx], Cs[buf][cy + 1][cx], Cs[buf][cy + 2][cx], eps);
-                }
-                Fy[ty][tx] = f;
-            }
-            // the tile's extra upper faces
-            if (ty == 0 && tx < kTY) {
-                T f = T(0);
-                if (!wall_xe) {
-                    const T uv = u[(kp + je_row) * a.nfx + fie];
-                    const int yy = tx + kHalo, xx = kTX + kHalo;
-                    f = face_flux(uv, Cs[buf][yy][xx - 3], Cs[buf][yy][xx - 2], Cs[buf][yy][xx - 1],
-                                  Cs[buf][yy][xx], Cs[buf][yy][xx + 1], Cs[buf][yy][xx + 2], eps);
-                }
-                Fx[tx][kTX] = f;
-            }
-            if (ty == 1) {
-                T f = T(0);
-                if (!wall_ye) {
-                    const T vv = v[((int64_t)k * a.nfy + fje) * a.nx + ic];
-                    const int yy = kTY + kHalo, xx = cx;
-                    f = face_flux(vv, Cs[buf][yy - 3][xx], Cs[buf][yy - 2][xx], Cs[buf][yy - 1][xx],
-                                  Cs[buf][yy][xx], Cs[buf][yy + 1][xx], Cs[buf][yy + 2][xx], eps);
-                }
-                Fy[kTY][tx] = f;
-            }
-            // z: flux through the upper face k+1 of this cell
-            {
-                const bool wall = (a.bcz != CH_PERIODIC) && (k + 1 >= a.nz);
-                if (!wall) {
-                    const int f = (k + 1 < a.nz) ? k + 1 : 0;
-                    const T wv = w[(int64_t)f * plane + col];
-                    fz_up = face_flux(wv, q[0], q[1], q[2], q[3], q[4], q[5], eps);
-                }
-            }
-            __syncthreads();
-        }
-
-        // M lap(psi'(C)), 7-point central (Sec. 3); neighbour differences are
-        // formed first, so FP32 keeps the accuracy of the small differences
-        const T c0 = Cs[buf][cy][cx];
-        const T pc = psi_p(c0);
-        T pzm = psi_p(q[1]), pzp = psi_p(q[3]);
-        if (a.bcz == CH_DIRICHLET) {  // the ghost of psi' is its own negated mirror (psi' = 0 on the wall)
-            if (k == 0) pzm = -psi_p(-q[1]);
-            if (k + 1 == a.nz) pzp = -psi_p(-q[3]);
-        }
-        const T lap = (((psi_p(Cs[buf][cy][cx - 1]) - pc) + (psi_p(Cs[buf][cy][cx + 1]) - pc)) +
-                       ((psi_p(Cs[buf][cy - 1][cx]) - pc) + (psi_p(Cs[buf][cy + 1][cx]) - pc)) +
-                       ((pzm - pc) + (pzp - pc))) *
-                      a.inv_h2;
-        // [1,-4,6,-4,1] sums of A_x + A_y + A_z (Eq. eq-a3d) as differences of
-        // second differences: D2(i-1) - 2 D2(i) + D2(i+1)
-        auto fourth = [&](T m2, T m1, T p1, T p2) {
-            const T da = m1 - c0, db = p1 - c0;
-            return ((m2 - m1) - da) + ((p2 - p1) - db) - T(2) * (da + db);
-        };
-        const T astar = fourth(Cs[buf][cy][cx - 2], Cs[buf][cy][cx - 1], Cs[buf][cy][cx + 1], Cs[buf][cy][cx + 2]) +
-                        fourth(Cs[buf][cy - 2][cx], Cs[buf][cy - 1][cx], Cs[buf][cy + 1][cx], Cs[buf][cy + 2][cx]) +
-                        fourth(q[0], q[1], q[3], q[4]);
-
-        T H = a.mob * lap;
-        if (ADV) {
-            const T div = (Fx[ty][tx + 1] - Fx[ty][tx]) + (Fy[ty + 1][tx] - Fy[ty][tx]) + (fz_up - fz_lo);
-            H -= div * a.inv_h;
-        }
-        if (in_xy) {
-            const int64_t idx = (int64_t)k * plane + (int64_t)j * a.nx + i;
-            T rhs = a.dtg * H - a.impl * astar;
-            if (a.has_prev) rhs += a.dtr * Hprev[idx];
-            Hout[idx] = H;
-            if (r) r[idx] = rhs;
-        }
-        // advance the z queue
-#pragma unroll
-        for (int m = 0; m < 5; ++m) q[m] = q[m + 1];
-        q[5] = qnext;
-        fz_lo = fz_up;
-    }
 }
 
 // ---------------------------------------------------------------------------
