@@ -1,8 +1,8 @@
-"""GPU tests of the marching line solver: one u = 0 step against the oracle
-where its blocks, restarts and ghost rows can go wrong (line lengths about the
-block sizes, lines shorter than the restart distance, every wall type, every
-copy width), for operators of each restart distance and for one that decays
-too slowly and takes the scan solvers."""
+"""GPU tests of the line solvers: one u = 0 step against the oracle where blocks,
+restarts and ghost rows can go wrong (line lengths about the block sizes, lines
+shorter than the restart distance, every wall type, every copy width), for
+operators of each restart distance and for one that decays too slowly and takes
+the scan solvers; and on boxes with lines enough for the streaming form."""
 import numpy as np
 import pytest
 
@@ -30,15 +30,32 @@ def _lib():
     capi.load()
 
 
+# boxes with more than 304 groups of 32 lines (1216 where rows are not 16-byte
+# aligned): the directions that stream, with a partial last block and last group
+STREAMED = [((104, 96, 72), "f32"),    # x, y
+            ((66, 100, 100), "f32"),   # z
+            ((200, 200, 67), "f32"),   # x unaligned
+            ((200, 70, 197), "f32"),   # y unaligned
+            ((70, 199, 197), "f32"),   # z unaligned
+            ((98, 100, 520), "f64")]   # x in FP64, too long for a tile
+
+
+@pytest.mark.parametrize("shape, prec", STREAMED)
+@pytest.mark.parametrize("bc", [(P, P, P), (N, N, D)])
+@pytest.mark.parametrize("ck", [0.25, 12.0])
+def test_streamed_lines_match_oracle(shape, prec, bc, ck):
+    test_one_step_matches_oracle(shape, ck, prec, bc)
+
+
 @pytest.mark.parametrize("prec", ["f64", "f32"])
 @pytest.mark.parametrize("shape", SHAPES)
 # ck of the first substep: restart distances of 1, 2 and 3 blocks, and the scan solvers
 @pytest.mark.parametrize("ck", [0.02, 1.2, 12.0, 400.0])
-def test_one_step_matches_oracle(shape, ck, prec):
+def test_one_step_matches_oracle(shape, ck, prec, bc=None):
     from paper_2105_01865_gb300.solver import Solver
     nz, ny, nx = shape
     h, cn, pe = 1.0 / 32, 0.75 / 32, 100.0
-    bc = BCS[(SHAPES.index(shape) + int(ck)) % len(BCS)]
+    bc = bc or BCS[(SHAPES.index(shape) + int(ck)) % len(BCS)]
     dt = ck / (8.0 / 15.0 / pe / 2.0 * 4.0 * cn ** 2 / h ** 4)
     rng = np.random.default_rng(nx)
     C0 = inputs.drops_field(shape, h, bc, [(nx * h / 2, ny * h / 3, nz * h / 2)], [0.3 * min(shape) * h], cn)
