@@ -197,7 +197,8 @@ int ch_free_energy(ch_handle* h, double* out);
 int ch_diagnostics(ch_handle* h, double* mass, double* free_energy);
 
 /* Wait for the handle's stream and report (then clear) the non-finite flag
- * (CH_ENONFINITE). */
+ * (CH_ENONFINITE).  CH_ETIMEOUT when a bounded wait between the warps of an
+ * explicit-kernel tile gave up (2 s); the step's results are then void. */
 int ch_sync(ch_handle* h);
 
 /* Number of kernel launches one ch_step(h, 1) enqueues. */

@@ -163,10 +163,10 @@ __device__ void run_phase(const BatchArgs& A, int ph, int l, float* smem) {
             float *Hp = B.H[(l + 1) & 1], *Ho = B.H[l & 1];
             if (B.rows == kRowsPeriodic)
                 explicit_tile3<false, false, kRowsPeriodic>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z,
-                                                            w.w, A.zchunk, sm);
+                                                            w.w, A.zchunk, sm, A.status);
             else
                 explicit_tile3<false, false, kRowsAny>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z, w.w,
-                                                       A.zchunk, sm);
+                                                       A.zchunk, sm, A.status);
         } else if (ph == 1) {
             switch (B.M[0]) {
                 case 1: x_item<1>(B, w.y, l); break;

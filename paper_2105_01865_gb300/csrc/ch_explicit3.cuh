@@ -6,11 +6,10 @@
 //
 // What bounds it: instruction issue, then the FMA pipe.  The paired arithmetic
 // of the formulas is about 180 instructions a pair and plane; what counts is
-// how many others come with it (442 instructions in all; 602 in the form this
-// replaces, at 5.36 against 4.85 ms a launch on 1024 x 1024 x 512, 1.43 against
-// 1.21 ms on 500^3 and, one cell a thread for odd nx, 81 against 56 us on
-// 211 x 157 x 93).  Issue stands at 55 %: a plane's barrier waits for the two
-// warps that also form the tile's extra faces.  So
+// how many others come with it (about 450 instructions in all; 602 in the form
+// this replaces, at 5.36 against 4.60 ms a launch on 1024 x 1024 x 512, 1.43
+// against 1.13 ms on 500^3 and, one cell a thread for odd nx, 81 against 57 us
+// on 211 x 157 x 93).  So
 //  - a plane's inputs arrive by asynchronous copies into shared memory, C as
 //    one 16-byte copy a thread, the face velocities and H^{l-1} as one 8-byte
 //    copy each into the thread's own slots, whose sources advance by one
@@ -19,7 +18,11 @@
 //  - a thread's x-window is four 8-byte shared loads; its upper x-face comes
 //    from the next lane by a shuffle; its lower faces stay in registers;
 //  - psi' is formed once a plane for the cell's own column and carried;
-//  - the WENO5 quotient is one reciprocal estimate.
+//  - the WENO5 quotient is one reciprocal estimate;
+//  - warps 0 and 1 also form the tile's extra faces, and the others need not wait
+//    for them at once: a warp arrives at a split barrier once its own x- and
+//    y-faces are published and waits after its z-faces, Laplacian and fourth
+//    differences (4.85 ms with one barrier in that place, 4.60 so).
 // 3 CTAs an SM at 80 registers (2 at 117: 4.91 ms); unaligned rows, which hold
 // more offsets, 2 at 120 (55 against 61 us on 211 x 157 x 93).
 // XM says how rows lie: kRowsPeriodic, 16-byte aligned (nx a multiple of 4) and
@@ -37,6 +40,37 @@ template <int N>
 __device__ __forceinline__ void cp_async_fill(float* smem, const float* gmem, int bytes) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gmem), "n"(N * 4), "r"(bytes) : "memory");
+}
+
+// Split barrier of a CTA's warps on a shared-memory mbarrier: a warp arrives
+// once its shared writes are done, works on, and waits later.  The wait gives up
+// after 2 s (false).
+__device__ __forceinline__ void warps_init(unsigned long long* bar, unsigned warps) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(warps)
+                 : "memory");
+}
+__device__ __forceinline__ void warps_arrive(unsigned long long* bar, int lane) {
+    __syncwarp();
+    if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
+}
+__device__ __forceinline__ bool warps_try(unsigned long long* bar, unsigned parity) {
+    unsigned ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok)
+                 : "r"((unsigned)__cvta_generic_to_shared(bar)), "r"(parity)
+                 : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool warps_wait(unsigned long long* bar, unsigned parity) {
+    if (warps_try(bar, parity)) return true;
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t0));
+    while (!warps_try(bar, parity)) {
+        asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
+        if (t - t0 > 2000000000ull) return false;
+    }
+    return true;
 }
 
 // WENO5 (Jiang-Shu) face values of two faces at once in first differences of
@@ -88,6 +122,7 @@ struct Explicit3Smem {
     __align__(16) float Sl[2][ADV ? 4 : 1][2 * NT];  // H^{l-1}, u, v, w of the thread's pair at [2 tid]
     __align__(16) float Sy[2][ADV ? kTX2 : 2];       // v of the tile's extra y-faces
     __align__(16) float Fy[ADV ? kTY + 1 : 1][kTX2];
+    unsigned long long bar;                          // split barrier of the face fluxes
     float Sx[2][ADV ? kTY : 1];                      // u of its extra x-faces
     float Fe[ADV ? kTY : 1];
     int gi_tab[PX], gj_tab[PY];
@@ -99,7 +134,8 @@ struct Explicit3Smem {
 template <bool ADV, bool DIRI, int XM>
 __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, const float* v, const float* w,
                                                const float* Hprev, float* Hout, float* r, const RhsArgs<float>& a,
-                                               int bx, int by, int bz, int zchunk, Explicit3Smem<ADV>& sm) {
+                                               int bx, int by, int bz, int zchunk, Explicit3Smem<ADV>& sm,
+                                               unsigned int* status) {
     constexpr int PX = kTX2 + 2 * kHL2, PY = kTY + 2 * kHalo, NT = 32 * kTY;
     constexpr bool AL = XM != kRowsAny, per_x = XM == kRowsPeriodic;  // per_x false: a.bcx decides
     constexpr int NB = Explicit3Smem<ADV>::NB;
@@ -129,6 +165,7 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
     };
 
     __syncthreads();  // the buffers may still be read by a previous tile of this CTA
+    if (ADV && tid == 0) warps_init(&sm.bar, kTY);
     if (tid < PX) gi_tab[tid] = bc_index(i0 + tid - kHL2, a.nx, a.bcx);
     else if (tid < PX + PY) gj_tab[tid - PX] = bc_index(j0 + (tid - PX) - kHalo, a.ny, a.bcy);
 
@@ -305,6 +342,9 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
                 Fe[2 * tx] = f.x();
                 Fe[2 * tx + 1] = f.y();
             }
+            // the face between this warp's rows and its neighbours' is published: arrive
+            // now, wait after the z-faces, the Laplacian and the fourth differences
+            warps_arrive(&sm.bar, tx);
             if (per_z || k + 1 < a.nz) fz_up = face_flux_q(ldp(S + 6 * NT), q[0], q[1], q[2], q[3], q[4], q[5], eps4);
         }
         // M lap(psi'(C)), neighbour differences first, so FP32 keeps the
@@ -326,7 +366,7 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
         Pr<float> H = mul(sp(a.mob), lap);
         if constexpr (ADV) {
             float fr = __shfl_down_sync(kFull, fx.x(), 1);  // the next lane's lower x-face
-            __syncthreads();
+            if (!warps_wait(&sm.bar, (k - k0) & 1)) atomicOr(status, 4u);
             if (tx == 31) fr = Fe[ty];
             const Pr<float> dxf = sub(mk(fx.y(), fr), fx), dyf = sub(ldp(&Fy[ty + 1][2 * tx]), fy);
             H = fma2(sp(-a.inv_h), add(add(dxf, dyf), sub(fz_up, fz_lo)), H);
@@ -362,11 +402,11 @@ template <bool ADV, bool DIRI, int XM>
 __global__ void __launch_bounds__(32 * kTY, XM == kRowsAny ? 2 : 3)
 ch_explicit_rhs3(const float* __restrict__ C, const float* __restrict__ u, const float* __restrict__ v,
                  const float* __restrict__ w, const float* __restrict__ Hprev, float* __restrict__ Hout,
-                 float* __restrict__ r, RhsArgs<float> a, int zchunk) {
+                 float* __restrict__ r, RhsArgs<float> a, int zchunk, unsigned int* status) {
     pdl_wait();
     pdl_launch_dependents();
     __shared__ Explicit3Smem<ADV> sm;
-    explicit_tile3<ADV, DIRI, XM>(C, u, v, w, Hprev, Hout, r, a, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, sm);
+    explicit_tile3<ADV, DIRI, XM>(C, u, v, w, Hprev, Hout, r, a, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, sm, status);
 }
 
 }  // namespace chg

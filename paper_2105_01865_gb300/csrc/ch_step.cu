@@ -853,7 +853,7 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
         auto go = [&](auto adv, auto dir, auto xmc) {
             // without H^{l-1} its copies have length 0: any valid source
             launch_k(h->stream, ch_explicit_rhs3<decltype(adv)::value, decltype(dir)::value, decltype(xmc)::value>, grid,
-                     block, 0, C, u, v, w, Hprev ? Hprev : C, Hout, r, a, tz);
+                     block, 0, C, u, v, w, Hprev ? Hprev : C, Hout, r, a, tz, h->status);
         };
         using Yes = std::true_type;
         using No = std::false_type;
@@ -1240,6 +1240,7 @@ int ch_sync(ch_handle* h) {
     if (flag) {
         CHG_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(unsigned int), h->stream));
         CHG_CUDA(h, cudaStreamSynchronize(h->stream));
+        if (flag & 4u) return fail(h, CH_ETIMEOUT, "a barrier of the explicit kernel did not complete");
         return fail(h, CH_ENONFINITE, "non-finite value in C");
     }
     return CH_OK;
