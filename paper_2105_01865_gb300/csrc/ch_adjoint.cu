@@ -34,31 +34,38 @@ struct AdjArgs {
 template <typename T>
 __device__ __forceinline__ T psi_prime_t(T c) { return c * (c * (c - T(1.5)) + T(0.5)); }
 
-// Sum of products for dL/dM.  FP64 fields multiply and add in FP64.  FP32
-// fields keep a double-float pair: the product's rounding error comes exactly
-// out of one fused multiply-add, the sum's out of TwoSum, so a thread's partial
-// sum is good to about 2^-48 of its terms without FP64 arithmetic, which would
-// bound the kernel (8 multiply-adds and 9 conversions a cell at 1/64 of the
-// FP32 rate).
-template <typename T>
-struct AdjDot {
-    T s = T(0);
-    __device__ __forceinline__ void add(T a, T b) { s += a * b; }
-    __device__ __forceinline__ double total() const { return s; }
-};
-template <>
-struct AdjDot<float> {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float x = __fmul_rn(a, b);
-        const float xe = __fmaf_rn(a, b, -x);
-        const float t = __fadd_rn(s, x);
-        const float bp = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(x, bp)), xe));
-        s = t;
-    }
-    __device__ __forceinline__ double total() const { return (double)s + (double)c; }
-};
+// The products of a cell for dL/dM, into FP64 sums: FP64 holds the product of two
+// FP32 values exactly and has range to spare for any scale of the loss.
+__device__ __forceinline__ void adj_dots(const double (&a)[5], const double (&b)[5], double& d1, double& d2) {
+    d1 += a[0] * b[0];
+#pragma unroll
+    for (int m = 1; m < 5; ++m) d2 += a[m] * b[m];
+}
+// FP32 values are widened by their bits on the integer pipe, and by the
+// conversion, which runs at 1/64 of the FP32 rate like the multiply-adds, only in
+// cells where one is subnormal or not finite.  128^3: a launch takes 69 us, 100
+// with conversions throughout, 50 with sums in double-float, which has no more than
+// FP32's range and 48 bits.
+__device__ __forceinline__ bool zero_or_normal(float f) {
+    const unsigned t = __float_as_uint(f) << 1;  // without its sign
+    return t == 0u || t - 0x01000000u < 0xfe000000u;
+}
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f);
+    const unsigned hi = ((unsigned)((int)b >> 3) & 0x8fffffffu) + 0x38000000u;  // exponent bias 127 -> 1023
+    return f == 0.f ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
+}
+__device__ __forceinline__ void adj_dots(const float (&a)[5], const float (&b)[5], double& d1, double& d2) {
+    bool plain = true;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) plain = plain & zero_or_normal(a[m]) & zero_or_normal(b[m]);
+    if (plain)
+        adj_dots({widen(a[0]), widen(a[1]), widen(a[2]), widen(a[3]), widen(a[4])},
+                 {widen(b[0]), widen(b[1]), widen(b[2]), widen(b[3]), widen(b[4])}, d1, d2);
+    else
+        adj_dots({(double)a[0], (double)a[1], (double)a[2], (double)a[3], (double)a[4]},
+                 {(double)b[0], (double)b[1], (double)b[2], (double)b[3], (double)b[4]}, d1, d2);
+}
 
 // [1,-4,6,-4,1] of five neighbours along one direction, as differences
 template <typename T>
@@ -72,10 +79,11 @@ __device__ __forceinline__ T fourth(T m2, T m1, T c, T p1, T p2) {
 // in-plane ones are read through offsets found once, so a cell costs 27 loads
 // that neighbouring threads share in L1.  Bound by those loads.  One thread a
 // cell, with every neighbour's index reduced modulo the box, took 356 us on
-// 128^3 (FP32); this form 50.
+// 128^3 (FP32); this form 69, 19 of them for the FP64 sums.  FP32 takes 4 CTAs an SM (64
+// registers; 3 at 76: 82 us).
 constexpr int kAdjZ = 8;
 template <typename T>
-__global__ void __launch_bounds__(kAThreadsX * kAThreadsY)
+__global__ void __launch_bounds__(kAThreadsX * kAThreadsY, sizeof(T) == 4 ? 4 : 2)
 adj_substep(const T* __restrict__ C, const T* __restrict__ lam_r, const T* __restrict__ lamH_in,
             const T* __restrict__ lamC_in, const T* __restrict__ s0, const T* __restrict__ s1,
             const T* __restrict__ s2, T* __restrict__ lamC_out, T* __restrict__ lamHp_out, double* partials,
@@ -102,7 +110,7 @@ adj_substep(const T* __restrict__ C, const T* __restrict__ lam_r, const T* __res
             ql[m] = lam_r[zoff(k0 - 2 + m)];
         }
         T hm = lamH_in[zoff(k0 - 1)], hc = lamH_in[zoff(k0)];
-        AdjDot<T> d1, d2;  // <lam_H, lap psi'> and <lam_r, A C> + sum_d <A_d lam_r, s_d> / 2
+        double d1 = 0.0, d2 = 0.0;  // <lam_H, lap psi'> and <lam_r, A C> + sum_d <A_d lam_r, s_d> / 2
         for (int k = k0; k < k1; ++k) {
             const int64_t e = k * plane + ij, z2 = zoff(k + 2);
             qc[4] = C[z2];
@@ -129,11 +137,8 @@ adj_substep(const T* __restrict__ C, const T* __restrict__ lam_r, const T* __res
             const T ppp = (T(3) * c - T(3)) * c + T(0.5);
             lamC_out[e] = lamC_in[e] - adt * mob * ((A_lr[0] + A_lr[1]) + A_lr[2]) + ppp * mob * lap_lh;
             lamHp_out[e] = dtr * lr;
-            d1.add(lh0, lap_psi);
-            d2.add(lr, A_C);
-            d2.add(T(0.5) * A_lr[0], s0[e]);
-            d2.add(T(0.5) * A_lr[1], s1[e]);
-            d2.add(T(0.5) * A_lr[2], s2[e]);
+            adj_dots({lh0, lr, T(0.5) * A_lr[0], T(0.5) * A_lr[1], T(0.5) * A_lr[2]}, {lap_psi, A_C, s0[e], s1[e], s2[e]}, d1,
+                     d2);
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 qc[m] = qc[m + 1];
@@ -142,7 +147,7 @@ adj_substep(const T* __restrict__ C, const T* __restrict__ lam_r, const T* __res
             hm = hc;
             hc = hp;
         }
-        dm = d1.total() - a.alpha * a.dt * d2.total();
+        dm = d1 - a.alpha * a.dt * d2;
     }
     __shared__ double ws[kAThreadsX * kAThreadsY / 32];
     for (int o = 16; o > 0; o >>= 1) dm += __shfl_xor_sync(0xffffffffu, dm, o);

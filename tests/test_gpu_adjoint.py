@@ -155,3 +155,27 @@ def test_autograd_function():
     lam0, dM = s.adjoint(C0, 7, (2 * h ** 3 * (CT.detach() - target)).cpu().numpy(), 3)
     assert torch.allclose(C0t.grad, lam0, rtol=0, atol=1e-14 * float(lam0.abs().max()))
     assert abs(float(M.grad) - dM) <= 1e-12 * abs(dM)
+
+
+# amplitude of C, power of two on lam_T: products of the two fields over FP32's
+# largest value, and in its subnormal range
+@pytest.mark.parametrize("amp, power", [(1.0, 20), (100.0, 112), (1e-14, -70)])
+def test_fp32_gradient_in_m_scales_with_the_loss(amp, power):
+    """lam_T times a power of two: every FP32 field of the reverse pass scales
+    exactly while it stays normal, so dL/dC0 and, summed in FP64, dL/dM do."""
+    from paper_2105_01865_gb300.solver import Solver
+    bc = (co.PERIODIC, co.PERIODIC, co.NOFLUX)
+    shape, rng = (10, 12, 14), np.random.default_rng(8)
+    C0 = amp * rng.standard_normal(shape)
+    lamT = rng.standard_normal(shape).astype(np.float32)
+    out = {}
+    for prec in ("f32", "f64"):
+        s = Solver(shape, 1.0, bc, 0.75, 1e6, 1.0, C0.astype(np.float32), precision=prec)
+        out[prec] = s.adjoint(C0.astype(np.float32), 1, lamT, 1)
+        if prec == "f32":
+            lam0, dM = s.adjoint(C0.astype(np.float32), 1, lamT * np.float32(2.0 ** power), 1)
+        s.close()
+    assert np.isfinite(dM) and dM == out["f32"][1] * 2.0 ** power
+    assert np.array_equal(lam0.cpu().numpy(), out["f32"][0].cpu().numpy() * np.float32(2.0 ** power))
+    # the bar of the FP32 adjoint test above
+    assert abs(out["f32"][1] - out["f64"][1]) <= 1e-4 * abs(out["f64"][1])
