@@ -24,10 +24,13 @@
 
 namespace chg {
 
-// a / b to within rounding: the hardware's reciprocal estimate (2^-20), one
-// Newton step (2^-40) and one correction of the quotient by its exact residual
-// (Markstein's scheme).  b is normal and positive here.
+// a / b to within a unit in the last place: the hardware's reciprocal estimate
+// (2^-20), one Newton step (2^-40) and one correction of the quotient by its
+// residual (Markstein's scheme).  Outside 2^-800 .. 2^1000, where b, its
+// reciprocal or the residual may be subnormal (the estimate takes a subnormal for
+// zero), the division.
 __device__ __forceinline__ double div_newton(double a, double b) {
+    if ((unsigned)__double2hiint(b) - 0x0df00000u > 0x7e700000u - 0x0df00000u) return a / b;
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
     y = fma(y, fma(-b, y, 1.0), y);

@@ -75,3 +75,71 @@ def test_fp32_two_steps_match_oracle(nx, bc, flow):
     ref = co.step(C0, vel, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=0.2 * h, bc=bc), 2)
     # the bar of the other FP32 tests of a few steps
     assert_parity(got, ref, 1e-6, f"FP32 explicit {shape} {bc} flow={flow}")
+
+
+DIV_PROBE = """
+#include "ch_explicit64.cuh"
+__global__ void div_kernel(const double* a, const double* b, double* q, long n) {
+    const long i = blockIdx.x * 256L + threadIdx.x;
+    if (i < n) q[i] = chg::div_newton(a[i], b[i]);
+}
+extern "C" int div_probe(const double* a, const double* b, double* q, long n) {
+    div_kernel<<<(unsigned)((n + 255) / 256), 256>>>(a, b, q, n);
+    return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+def test_weno_quotient_is_a_division(tmp_path):
+    """The FP64 WENO5 quotient over every exponent a sum of weights can have: within a unit in the last
+    place of a / b, and the same as a / b where b or its reciprocal is near the subnormals, or not a number."""
+    import ctypes
+    import subprocess
+    from paper_2105_01865_gb300 import build
+    src, lib = tmp_path / "div.cu", tmp_path / "libdiv.so"
+    src.write_text(DIV_PROBE)
+    subprocess.run(["nvcc", *build.ARCH, *build.FLAGS, "-I", build.CSRC, "-shared", str(src), "-o", str(lib)], check=True)
+    rng = np.random.default_rng(1)
+    with np.errstate(all="ignore"):
+        e = np.concatenate([rng.uniform(-1074, 1023, 200_000), np.repeat([-1074, -1023, -1022, -801, -800, -799, 999, 1000,
+                                                                         1001, 1022, 1023], 2000).astype(float)])
+        b = np.ldexp(rng.uniform(1, 2, e.size), e.astype(int))
+        g = np.ldexp(rng.uniform(-2, 2, e.size), rng.integers(-60, 1, e.size))  # the quotient: differences of C
+        a = b * g
+        edge = np.array([0.0, -0.0, np.inf, np.nan, 5e-324, 2.0 ** -1022, 1.0])
+        a, b = np.append(a, np.repeat(edge, edge.size)), np.append(b, np.tile(edge, edge.size))
+        ref = a / b
+    ta, tb = torch.tensor(a, device="cuda"), torch.tensor(b, device="cuda")
+    tq = torch.empty_like(ta)
+    fn = ctypes.CDLL(str(lib)).div_probe
+    fn.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_long]
+    torch.cuda.synchronize()
+    assert fn(ta.data_ptr(), tb.data_ptr(), tq.data_ptr(), ta.numel()) == 0
+    q = tq.cpu().numpy()
+    near = (b >= 2.0 ** -799) & (b < 2.0 ** 1000)
+    assert np.array_equal(q[~near & (b < 2.0 ** -800)], ref[~near & (b < 2.0 ** -800)], equal_nan=True)
+    assert np.array_equal(q[b >= 2.0 ** 1001], ref[b >= 2.0 ** 1001], equal_nan=True)
+    assert np.array_equal(q[np.isnan(b)], ref[np.isnan(b)], equal_nan=True)
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(q), fin)
+    ulps = np.abs(q[fin] - ref[fin]) / np.spacing(np.abs(ref[fin]))
+    print(f"quotient: at most {ulps.max():.0f} units in the last place from a / b, {np.mean(ulps > 0):.1e} of them not equal")
+    assert ulps.max() <= 1
+
+
+# a regulariser whose fourth power is subnormal or zero in the weights of a constant region
+@pytest.mark.parametrize("weno_eps", [1e-6, 1e-79, 1e-80])
+def test_fp64_small_regulariser(weno_eps):
+    from paper_2105_01865_gb300.solver import Solver
+    shape, bc, h, cn, pe = (9, 12, 40), (P, N, N), 1.0 / 16, 0.75 / 16, 20.0
+    C0 = np.zeros(shape)
+    C0[:, :, 12:20] = 1.0  # constant on both sides
+    vel = inputs.curl_velocity(*(inputs.uniform_faces(n, n * h) for n in shape[::-1]), bc, seed=5, kmax=3)
+    s = Solver(shape, h, bc, cn, pe, 0.2 * h, C0, precision="f64", weno_eps=weno_eps, advect=True)
+    s.set_velocity_fine(*vel)
+    s.step(1)
+    got = s.field()
+    s.close()
+    nz, ny, nx = shape
+    p = co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=0.2 * h, bc=bc, eps=weno_eps)
+    assert_parity(got, co.step(C0, vel, p, 1), 1e-12, f"weno_eps {weno_eps}")
