@@ -51,7 +51,7 @@ struct BoxDesc {
     // 0 where the line is too long and the shared-memory tile solver runs
     int colR[2];
     CCoef<float> cols[2][kRK];
-    int rows;  // kRowsAny, kRowsWalled or kRowsPeriodic
+    int rows;  // kRowsPeriodic where rows are 16-byte aligned and periodic, else kRowsEven (nx is even)
 };
 
 struct BatchArgs {
@@ -165,8 +165,8 @@ __device__ void run_phase(const BatchArgs& A, int ph, int l, float* smem) {
                 explicit_tile3<false, false, kRowsPeriodic>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z,
                                                             w.w, A.zchunk, sm, A.status);
             else
-                explicit_tile3<false, false, kRowsAny>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z, w.w,
-                                                       A.zchunk, sm, A.status);
+                explicit_tile3<false, false, kRowsEven>(B.C, nullptr, nullptr, nullptr, Hp, Ho, B.r, B.rhs[l], w.y, w.z, w.w,
+                                                        A.zchunk, sm, A.status);
         } else if (ph == 1) {
             switch (B.M[0]) {
                 case 1: x_item<1>(B, w.y, l); break;
@@ -498,7 +498,7 @@ int ch_batch_create(const ch_params* boxes, int nbox, void* const* C, void* work
         B.ny = (int)p.ny;
         B.nz = (int)p.nz;
         B.nlines_x = (int)(p.ny * p.nz);
-        B.rows = p.nx % 4 == 0 && p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsAny;
+        B.rows = p.nx % 4 == 0 && p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsEven;
         const double mob = 1.0 / p.pe;
         const double kappa = p.w * p.cn * p.cn / (p.h * p.h * p.h * p.h);
         for (int l = 0; l < kRK; ++l) {

@@ -23,12 +23,14 @@
 //    for them at once: a warp arrives at a split barrier once its own x- and
 //    y-faces are published and waits after its z-faces, Laplacian and fourth
 //    differences (4.85 ms with one barrier in that place, 4.60 so).
-// 3 CTAs an SM at 80 registers (2 at 117: 4.91 ms); unaligned rows, which hold
+// 3 CTAs an SM at 80 registers (2 at 117: 4.91 ms); odd rows, which hold
 // more offsets, 2 at 120 (55 against 61 us on 211 x 157 x 93).
 // XM says how rows lie: kRowsPeriodic, 16-byte aligned (nx a multiple of 4) and
 // periodic, so that a halo chunk is a chunk of the row's other end; kRowsWalled,
-// aligned with walls; kRowsAny, nx of any kind, odd too: copies, loads and stores
-// go element by element.
+// aligned with walls; kRowsEven, nx even: pairs of cells are 8-byte aligned, whole
+// and never wrap, so everything but u moves in pairs (198 x 200 x 150: 93 us, 117 as
+// kRowsAny; 514 x 130 x 66: 68 and 86); kRowsAny, odd rows: copies, loads and stores go
+// element by element.
 #pragma once
 
 #include "ch_pairs.cuh"
@@ -110,7 +112,7 @@ __device__ __forceinline__ Pr<float> face_flux_q(Pr<float> vel, Pr<float> m3, Pr
                            mk(ux ? p1.x() : m2.x(), uy ? p1.y() : m2.y()), eps4));
 }
 
-enum { kRowsAny, kRowsWalled, kRowsPeriodic };
+enum { kRowsAny, kRowsEven, kRowsWalled, kRowsPeriodic };
 
 template <bool ADV>
 struct Explicit3Smem {
@@ -137,7 +139,8 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
                                                int bx, int by, int bz, int zchunk, Explicit3Smem<ADV>& sm,
                                                unsigned int* status) {
     constexpr int PX = kTX2 + 2 * kHL2, PY = kTY + 2 * kHalo, NT = 32 * kTY;
-    constexpr bool AL = XM != kRowsAny, per_x = XM == kRowsPeriodic;  // per_x false: a.bcx decides
+    // AL: rows are 16-byte aligned; EV: 8-byte aligned, so both cells of a pair are in or out
+    constexpr bool EV = XM != kRowsAny, AL = EV && XM != kRowsEven, per_x = XM == kRowsPeriodic;  // per_x false: a.bcx decides
     constexpr int NB = Explicit3Smem<ADV>::NB;
     auto& Cs = sm.Cs;
     auto& Sl = sm.Sl;
@@ -151,16 +154,16 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
     const int tid = threadIdx.x + threadIdx.y * 32, tx = tid & 31, ty = tid >> 5;
     const int i0 = bx * kTX2, j0 = by * kTY, k0 = bz * zchunk, kend = min(k0 + zchunk, a.nz);
     const int ia = i0 + 2 * tx, j = j0 + ty;
-    const bool in_a = ia < a.nx && j < a.ny, in_b = AL ? in_a : ia + 1 < a.nx && j < a.ny;
+    const bool in_a = ia < a.nx && j < a.ny, in_b = EV ? in_a : ia + 1 < a.nx && j < a.ny;
     // the pair's columns in global memory; where the second is past the row, the
     // one that its ghost copies
-    const int jc = min(j, a.ny - 1), ic = min(ia, AL ? a.nx - 2 : a.nx - 1);
-    const int icb = AL || ic + 1 < a.nx ? ic + 1 : (a.bcx == CH_PERIODIC ? 0 : a.nx - 1);
+    const int jc = min(j, a.ny - 1), ic = min(ia, EV ? a.nx - 2 : a.nx - 1);
+    const int icb = EV || ic + 1 < a.nx ? ic + 1 : (a.bcx == CH_PERIODIC ? 0 : a.nx - 1);
     const int plane = a.nx * a.ny;  // every field holds fewer than 2^31 elements
     const int col = jc * a.nx + ic;
     const Pr<float> eps4 = sp(4.f * a.eps);
     auto ld2g = [&](const float* p) {  // the pair whose first element is at column ic
-        if constexpr (AL) return ldp(p);
+        if constexpr (EV) return ldp(p);
         else return mk(p[0], p[icb - ic]);
     };
 
@@ -188,9 +191,10 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
 
     // this thread's copies.  C: AL, chunk tid of 252 (18 a row; the last threads
     // repeat the last one); a chunk past a no-flux x-wall is reversed, element by
-    // element.  Else elements tid + 256 m.
+    // element.  EV, pairs likewise: pairs tid and tid + 256 of 504 (36 a row).  Else
+    // elements tid + 256 m.
     const int ctid = min(tid, PX * PY / 4 - 1);
-    constexpr int kCN = AL ? 1 : (PX * PY + NT - 1) / NT;
+    constexpr int kCN = AL ? 1 : EV ? 2 : (PX * PY + NT - 1) / NT;
     int csrc[kCN];
     bool rev = false;
     if constexpr (AL) {
@@ -198,6 +202,15 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
         rev = !per_x && (c0 < 0 || c0 == a.nx);
         // chunks further past a wall are never used: any valid source
         csrc[0] = gj_tab[row] * a.nx + (!per_x && c0 > a.nx ? 0 : gi_tab[c]);
+    } else if constexpr (EV) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int e = min(tid + m * NT, PX * PY / 2 - 1), row = e / (PX / 2), c = (e - row * (PX / 2)) * 2;
+            const int c0 = i0 + c - kHL2;
+            const bool wall = a.bcx != CH_PERIODIC;
+            csrc[m] = gj_tab[row] * a.nx + (wall && c0 > a.nx + 2 ? 0 : gi_tab[c]);
+            if (wall && (c0 < 0 || c0 == a.nx || c0 == a.nx + 2)) csrc[m] = ~csrc[m];  // reversed
+        }
     } else {
 #pragma unroll
         for (int m = 0; m < kCN; ++m) {
@@ -248,13 +261,24 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
             else
 #pragma unroll
                 for (int e = 0; e < 4; ++e) cp_async_elem(dst + 4 * ctid + e, Ck + csrc[0] - e);
+        } else if constexpr (EV) {
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                float* d = dst + 2 * min(tid + m * NT, PX * PY / 2 - 1);
+                if (csrc[m] >= 0) {
+                    cp_async_pair(d, Ck + csrc[m]);
+                } else {
+                    cp_async_elem(d, Ck + ~csrc[m]);
+                    cp_async_elem(d + 1, Ck + (~csrc[m] - 1));
+                }
+            }
         } else {
 #pragma unroll
             for (int m = 0; m < kCN; ++m)
                 if (tid + m * NT < PX * PY) cp_async_elem(dst + tid + m * NT, Ck + csrc[m]);
         }
         float* S = slot + s * SB;
-        if constexpr (AL) {
+        if constexpr (EV) {
             cp_async_fill<2>(S, Hprev + eh, 2 * nh);
         } else {
             cp_async_fill<1>(S, Hprev + eh, nh);
@@ -270,7 +294,7 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
             }
             // the z-face above plane kk: w of plane kk + 1, wrapped
             const float* wk = w + (kk + 1 < a.nz || !per_z ? ew + plane : col);
-            if constexpr (AL) {
+            if constexpr (EV) {
                 cp_async_fill<2>(S + 4 * NT, v + ev, 2 * nv);
                 cp_async_pair(S + 6 * NT, wk);
             } else {
@@ -280,7 +304,7 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
                 cp_async_elem(S + 6 * NT + 1, wk + (icb - ic));
             }
             if (ty == 0) {
-                if constexpr (AL) {
+                if constexpr (EV) {
                     cp_async_fill<2>(&Sy[s][2 * tx], v + ex, 2 * nx_);
                 } else {
                     cp_async_fill<1>(&Sy[s][2 * tx], v + ex, nx_);
@@ -373,7 +397,7 @@ __device__ __forceinline__ void explicit_tile3(const float* C, const float* u, c
             fz_lo = fz_up;
         }
         const Pr<float> rhs = fma2(sp(a.dtr), hp, fma2(sp(-a.impl), astar, mul(sp(a.dtg), H)));
-        if constexpr (AL) {
+        if constexpr (EV) {
             if (in_a) {
                 stp(Hout + idx, H);
                 if (r) stp(r + idx, rhs);

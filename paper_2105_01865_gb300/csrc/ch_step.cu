@@ -847,7 +847,7 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
     } else {
         const bool diri = p.bc[2] == CH_DIRICHLET;
         const int64_t xy = (int64_t)((nx + kTX2 - 1) / kTX2) * ((ny + kTY - 1) / kTY);
-        const int xm = nx % 4 ? kRowsAny : p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsWalled;
+        const int xm = nx % 2 ? kRowsAny : nx % 4 ? kRowsEven : p.bc[0] == CH_PERIODIC ? kRowsPeriodic : kRowsWalled;
         const int tz = explicit_depth(xy, nz, 152 * (xm == kRowsAny ? 2 : 3));
         const dim3 grid((nx + kTX2 - 1) / kTX2, (ny + kTY - 1) / kTY, (nz + tz - 1) / tz), block(32, kTY);
         auto go = [&](auto adv, auto dir, auto xmc) {
@@ -865,6 +865,7 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
         };
         if (xm == kRowsPeriodic) go2(std::integral_constant<int, kRowsPeriodic>{});
         else if (xm == kRowsWalled) go2(std::integral_constant<int, kRowsWalled>{});
+        else if (xm == kRowsEven) go2(std::integral_constant<int, kRowsEven>{});
         else go2(std::integral_constant<int, kRowsAny>{});
     }
     CHG_CUDA(h, cudaGetLastError());

@@ -143,3 +143,42 @@ def test_fp64_small_regulariser(weno_eps):
     nz, ny, nx = shape
     p = co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=0.2 * h, bc=bc, eps=weno_eps)
     assert_parity(got, co.step(C0, vel, p, 1), 1e-12, f"weno_eps {weno_eps}")
+
+
+def depth_fp32(nx, ny, nz, slots):
+    """Planes a FP32 tile marches (explicit_depth in ch_step.cu): the depth whose waves take the least."""
+    xy, best = -(-nx // 64) * -(-ny // 8), None
+    for c in range(1, nz + 1):
+        tz = -(-nz // c)
+        cost = -(-(xy * -(-nz // tz)) // slots) * (tz + 2.0)
+        if best is None or cost < best[0]:
+            best = (cost, tz)
+    return best[1]
+
+
+# rows of any kind, even rows, aligned rows with walls and without; tiles of several planes, the last one shorter
+@pytest.mark.parametrize("nx", [67, 66, 68])
+@pytest.mark.parametrize("bc", [(P, P, P), (N, P, P), (N, N, N), (P, P, N), (P, N, D), (N, P, D)])
+@pytest.mark.parametrize("flow", [True, False])
+def test_fp32_deep_tiles_match_oracle(nx, bc, flow):
+    from paper_2105_01865_gb300.solver import Solver
+    nz, ny = 11, 597
+    for slots in (2 * 152, 3 * 152):
+        tz = depth_fp32(nx, ny, nz, slots)
+        assert tz >= 3 and nz % tz != 0
+    h, cn, pe = 1.0 / 16, 0.75 / 16, 20.0
+    rng = np.random.default_rng(nx)
+    C0 = (0.5 + 0.4 * rng.standard_normal((nz, ny, nx))).astype(np.float32).astype(np.float64)
+    vel = None
+    if flow:
+        vel = inputs.curl_velocity(*(inputs.uniform_faces(n, n * h) for n in (nx, ny, nz)), bc, seed=nx, kmax=3)
+        vel = [a.astype(np.float32).astype(np.float64) for a in vel]
+    s = Solver((nz, ny, nx), h, bc, cn, pe, 0.2 * h, C0, precision="f32", advect=flow)
+    if flow:
+        s.set_velocity_fine(*vel)
+    s.step(1)
+    got = s.field()
+    s.close()
+    ref = co.step(C0, vel, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=0.2 * h, bc=bc), 1)
+    # the bar of the other FP32 tests of a few steps
+    assert_parity(got, ref, 1e-6, f"FP32 deep tiles nx={nx} {bc} flow={flow}")
