@@ -114,3 +114,19 @@ def test_full_size_shear_drop_one_step():
     ref = co.step_standard(f["C"].astype(np.float32).astype(np.float64), f["vel"],
                            params(f["shape"], h, f["bc"], f["cn"], f["pe"], dt), 1)
     assert_parity(s.field(), ref, 1e-6, "FP32 standard scheme 256x256x128, 1 step")
+
+
+# FP32 rows of 2 to 33 quads: blocks of 8, 16 and 32 quads by 32, 16 and 8 rows, the last of each partial
+@pytest.mark.parametrize("nx", [8, 32, 36, 68, 132])
+@pytest.mark.parametrize("ny", [7, 35])
+@pytest.mark.parametrize("bc", [(co.PERIODIC,) * 3, (co.NOFLUX, co.PERIODIC, co.NOFLUX)])
+def test_fp32_quads_match_oracle(nx, ny, bc):
+    shape = (6, ny, nx)
+    h, cn, pe, dt, C0, vel = case(shape, bc, nx, True)
+    C0 = C0.astype(np.float32).astype(np.float64)
+    vel = [a.astype(np.float32).astype(np.float64) for a in vel]
+    s = make(shape, h, bc, cn, pe, dt, C0, "f32", vel)
+    s.step(3)
+    got = s.field()
+    s.close()
+    assert_parity(got, co.step_standard(C0, vel, params(shape, h, bc, cn, pe, dt), 3), 1e-5, f"standard {shape} {bc}")
