@@ -293,7 +293,7 @@ def measured_peak_hbm():
 # the sources the step kernels (explicit right-hand side, x, y, z solves) are
 # built from: a change to any of them voids the recorded DRAM traffic
 STEP_SOURCES = ["ch_step.cu", "ch_kernels.cuh", "ch_pairs.cuh", "ch_explicit3.cuh", "ch_explicit64.cuh", "ch_march.cuh",
-                "ch_cols2.cuh", "line_tables.h", "ch_internal.h"]
+                "ch_cols2.cuh", "line_rule.h", "line_tables.h", "ch_internal.h"]
 
 
 def kernel_source_sha():

@@ -12,8 +12,9 @@
 // below 2^-36 (FP32) or 2^-64 (FP64) of the solution, under its rounding by
 // 2^12 and 2^11.  So the upward pass starts kb blocks before the line, on
 // ghost rows, and the downward pass of each block of B rows starts kb blocks
-// above it.  Operators that decay more slowly (over kMarchMaxReach rows) keep the
-// scan solvers of ch_kernels.cuh and ch_cols2.cuh.
+// above it.  Operators that decay more slowly (over kMarchMaxReach rows) and lines
+// no longer than their kb blocks keep the scan solvers of ch_kernels.cuh and
+// ch_cols2.cuh; between the forms that take a line, line_rule.h chooses.
 //
 // A warp streams its lines through a ring of shared-memory blocks: block b is
 // being swept upward while blocks b + 1 .. b + D are in flight (cp.async) and
@@ -34,18 +35,9 @@
 #include <type_traits>
 
 #include "ch_kernels.cuh"
+#include "line_rule.h"
 
 namespace chg {
-
-constexpr int kMarchMaxReach = 96;  // rows
-
-template <typename T>
-struct MarchShape {  // rows per block, blocks in flight
-    static constexpr int B = sizeof(T) == 4 ? 32 : 64;
-    // FP32, 1 and 3 blocks in flight: x 697 and 682 us against 675, z 1083 and
-    // 1092 against 1060 on 1024 x 1024 x 512
-    static constexpr int D = sizeof(T) == 4 ? 2 : 1;
-};
 
 template <typename T>
 struct MarchCoef {
@@ -55,17 +47,6 @@ struct MarchCoef {
     int reach;         // restart distance in rows (a multiple of 8)
     int kb;            // and in blocks of B rows (>= 1)
 };
-template <typename T>
-constexpr int march_max_kb() { return (kMarchMaxReach + MarchShape<T>::B - 1) / MarchShape<T>::B; }
-
-// The row that row j of the continued line copies; neg: with its sign flipped.
-__device__ __forceinline__ int march_row(int j, int n, int bc, bool& neg) {
-    const int p = bc == CH_PERIODIC ? n : 2 * n;
-    int m = j % p;
-    if (m < 0) m += p;
-    neg = bc == CH_DIRICHLET && m >= n;
-    return m < n ? m : 2 * n - 1 - m;
-}
 
 // V adjacent lines of one thread
 template <typename T, int V>
@@ -220,7 +201,7 @@ __device__ __forceinline__ void march_yz(const T* src, T* dst, T* Cf, int nc, in
     constexpr int CW = 32 * V, SLOT = B * CW;
     const int lane = threadIdx.x & 31;
     const int n = k.n, kb = k.kb, S = kb + 1 + D, cap = kb * B;
-    const bool per = k.bc == CH_PERIODIC, full = n <= cap;
+    const bool per = k.bc == CH_PERIODIC;
     T* save = sm + S * SLOT + V * lane;
     // copies: CPR of VL elements make a row, a warp copies RPI rows at once,
     // a block in B / RPI; this lane's column and first row
@@ -240,7 +221,7 @@ __device__ __forceinline__ void march_yz(const T* src, T* dst, T* Cf, int nc, in
             const int j0 = (b - kb) * B;  // first row of the block
             T* s = sm + o_load + r * CW + c;
             if (c < nc) {
-                if (j0 >= 0 || (per && !full)) {
+                if (j0 >= 0 || per) {
                     const T* g = src + (int64_t)(j0 + r + (j0 < 0 ? n : 0)) * ls + c;
                     if (j0 + B <= n) {
 #pragma unroll 8
@@ -249,11 +230,7 @@ __device__ __forceinline__ void march_yz(const T* src, T* dst, T* Cf, int nc, in
                         for (int i = 0; i + r < n - j0; i += RPI) march_copy<T, VL>(s + i * CW, g + i * ls);
                     }
                 } else {
-                    for (int i = 0; i < B; i += RPI) {
-                        bool neg;
-                        const int j = j0 + r + i;
-                        if (j < n) march_copy<T, VL>(s + i * CW, src + (full ? march_row(j, n, k.bc, neg) : -1 - j) * ls + c);
-                    }
+                    for (int i = 0; i < B; i += RPI) march_copy<T, VL>(s + i * CW, src + (-1 - j0 - r - i) * ls + c);
                 }
             }
         }
@@ -281,24 +258,6 @@ __device__ __forceinline__ void march_yz(const T* src, T* dst, T* Cf, int nc, in
     auto up = [&](int b) {
         const int j0 = (b - kb) * B;
         T* s = sm + o_up + V * lane;
-        if (full) {  // lines shorter than the restart distance: their copies wrap more than once
-            for (int i = 0; i < B; ++i) {
-                const int j = j0 + i;
-                L v = L::zero();
-                bool neg = false;
-                if (j < n + cap) {
-                    const int m = march_row(j, n, k.bc, neg);
-                    v = L::ld(j < n ? s + i * CW : save + m * CW);
-                    if (j >= 0 && j < n) v.st(save + j * CW);
-                    if (neg) v = v.neg();
-                }
-                const L y = lfma(k.nl1, y1, lfma(k.nl2, y2, v));
-                y2 = y1;
-                y1 = y;
-                lmul(k.dinv, y).st(s + i * CW);
-            }
-            return;
-        }
         if (j0 < 0 && k.bc == CH_DIRICHLET) return sweep(Some{}, No{}, Yes{}, s, s, s, 0, B);
         if (per && j0 >= 0 && j0 < cap) return sweep(Some{}, Yes{}, No{}, s, s, save + j0 * CW, CW, B);
         if (j0 < 0 || j0 + B <= (per ? n : n - cap)) return sweep(All{}, No{}, No{}, s, s, s, 0, B);
@@ -328,7 +287,8 @@ __device__ __forceinline__ void march_yz(const T* src, T* dst, T* Cf, int nc, in
     for (int b = 0; b < nb; ++b) {
         __syncwarp();  // the ring slot of block b + D has been read
         load(b + D);
-        // the block that is complete after this one's upward sweep, and its C
+        // the block that is complete after this one's upward sweep, and its C (FP64: 64
+        // rows, 424 bytes of which spill)
         const int t = b - kb, rows = min(B, n - (t - kb) * B);
         const int64_t row0 = (int64_t)((t - kb) * B) * ls;
         L cv[UPD ? B : 1];
@@ -413,7 +373,7 @@ __device__ __forceinline__ void march_x(const T* src, T* dst, int nl, const Marc
     constexpr int P = B + VEC, SLOT = 32 * P, CPL = B / VEC;
     const int lane = threadIdx.x & 31;
     const int n = k.n, kb = k.kb, S = kb + 1 + D, cap = kb * B;
-    const bool per = k.bc == CH_PERIODIC, full = n <= cap;
+    const bool per = k.bc == CH_PERIODIC;
     T* save = sm + S * SLOT + lane * (cap + VEC);
     const int nb = 2 * kb + (n + B - 1) / B;
     const int ring = S * SLOT;
@@ -429,7 +389,7 @@ __device__ __forceinline__ void march_x(const T* src, T* dst, int nl, const Marc
         if (b < nb) {
             const int j0 = (b - kb) * B;
             T* s = sm + o_load;
-            if (vec && (j0 >= 0 || (per && !full))) {
+            if (vec && (j0 >= 0 || per)) {
                 const T* g = src + first + j0 + (j0 < 0 ? n : 0);
                 s += l0 * P + c0;
                 if (nl == 32 && j0 + B <= n) {
@@ -440,10 +400,9 @@ __device__ __forceinline__ void march_x(const T* src, T* dst, int nl, const Marc
                 }
             } else {
                 for (int c = lane; c < B; c += 32) {
-                    bool neg;
                     const int j = j0 + c;
                     if (j < n) {
-                        const T* g = src + (j >= 0 ? j : full ? march_row(j, n, k.bc, neg) : per ? j + n : -1 - j);
+                        const T* g = src + (j >= 0 ? j : per ? j + n : -1 - j);
 #pragma unroll 4
                         for (int l = 0; l < nl; ++l) march_copy<T, 1>(s + l * P + c, g + (int64_t)l * n);
                     }
@@ -476,19 +435,7 @@ __device__ __forceinline__ void march_x(const T* src, T* dst, int nl, const Marc
     auto up = [&](int b) {
         const int j0 = (b - kb) * B;
         T* s = sm + o_up + lane * P;
-        if (full) {  // lines shorter than the restart distance: their copies wrap more than once
-            for (int i = 0; i < B; ++i) {
-                const int j = j0 + i;
-                T v = T(0);
-                bool neg;
-                if (j < n + cap) {
-                    const int m = march_row(j, n, k.bc, neg);
-                    v = j < n ? s[i] : save[m];
-                    if (j >= 0 && j < n) save[j] = v;
-                }
-                s[i] = row(v);
-            }
-        } else if (j0 + B <= (per || j0 < 0 ? n : n - cap)) {
+        if (j0 + B <= (per || j0 < 0 ? n : n - cap)) {
             if (per && j0 >= 0 && j0 < cap) sweep(std::true_type{}, s, s, save + j0);
             else sweep(std::false_type{}, s, s, s);
         } else if (vec && j0 >= n && j0 + B <= n + cap) {
@@ -605,19 +552,6 @@ ch_march_x(const T* src, T* dst, int64_t nlines, MarchCoef<T> k) {
 // streaming one and chains of only reach + R rows, for boxes too small to
 // fill the chip with one warp per 32 lines.  Needs reach <= n.
 // ---------------------------------------------------------------------------
-// Most warps of a CTA: what leaves a thread room for its R rows (and R of C).
-template <int R>
-constexpr int tile_max_warps() { return R <= 16 ? 20 : R <= 32 ? 16 : 8; }
-template <int R>
-__host__ __device__ constexpr int tile_warps(int n, int reach) { return (n + reach + R - 1) / R; }
-template <typename T, int R>
-__host__ __device__ constexpr size_t tile_yz_bytes(int warps) { return (size_t)warps * R * 32 * sizeof(T); }
-// x: the pitch keeps 16-byte accesses of adjacent lines free of bank conflicts
-template <typename T, int R>
-__host__ __device__ constexpr int tile_x_pitch(int warps) { return (warps * R + 31) / 32 * 32 + 16 / (int)sizeof(T); }
-template <typename T, int R>
-__host__ __device__ constexpr size_t tile_x_bytes(int warps) { return (size_t)tile_x_pitch<T, R>(warps) * 32 * sizeof(T); }
-
 // Row of the line that row j of its continuation copies, -n <= j < 2n.
 __device__ __forceinline__ int tile_row(int j, int n, bool per) {
     return j < 0 ? (per ? j + n : -1 - j) : j >= n ? (per ? j - n : 2 * n - 1 - j) : j;

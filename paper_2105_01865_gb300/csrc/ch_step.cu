@@ -19,6 +19,7 @@
 #include "ch_kernels.cuh"
 #include "ch_cols2.cuh"
 #include "ch_march.cuh"
+#include "line_rule.h"
 #include "line_tables.h"
 
 using namespace chg;
@@ -26,7 +27,6 @@ using namespace chg;
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory per CTA (sm_103a)
 
 // Use the two-column form of the column solver when nx is even, and its
 // cluster form for y/z lines longer than 256 cells.
@@ -530,51 +530,10 @@ bool multi_line_any(const ch_handle* h, int l, int dir) {
     }
 }
 
-// Which form solves the lines of dir.  Measured per launch (us, launch gap
-// included; old: the scan solvers) on boxes nx x ny x nz, x / y / z:
-//   FP32  256 x 256 x 1    old  8.3 14.2  -    tile16  8.4  8.9  -    march 10.4 12.5  -
-//         96^3             old 10.3 12.4 10.7  tile16  8.6  8.6 10.5  march  8.3 10.1 11.2
-//         128^3            old 12.4 12.4 14.4  tile16 11.6 11.7 12.6  march 10.0 10.3 11.5
-//         256 x 256 x 128  old 29.0 39.8 30.0  tile16 26.7 25.2 33.0  march 16.4 16.4 24.9
-//         211 x 157 x 93   old 18.9 33.1 29.9  tile32 14.6 16.5 16.7  march 18.4 18.5 22.5
-//         500^3            old  311  356  390                         march  177  170  343
-//         1024 x 1024 x 512  old 1280 1420 1390                       march  663  648 1060
-//         1000 x 100 x 60, x only: old 26.4, march 36.9 (188 warps of 1000 rows)
-//   FP64  64^3             old   35   25   25  tile32   22   23   26  tile64   29   31   37
-//         128^3            old  140  111  121  tile32   73   76   86  tile64   62   68   77  march 104 113 136
-//         256 x 256 x 128  old  382  444  369  tile32  218  217  266  tile64  201  222  252  march 258 281 359
-//         200^3            old  465  629  587  tile32  203  229  254  tile64  176  198  227
-// So: the scan solvers where the operator decays too slowly, the restart is
-// longer than the line, or the line is short (whole steps with u = 0: FP32 64^3
-// old 59 us, new 70; 80^3 84 and 78; 128^3 113 and 92; FP64 64^3 471 and 436).  FP64, bound by its arithmetic, takes the form with the fewest
-// restarts that still leaves every SM some warps: 64 rows a warp from 3
-// 32-line groups an SM on, else 32, where the line fits.  FP32 streams (march) once
-// 32-line groups outnumber the SMs two to one; fewer take 16 rows a warp, to
-// have warps enough; lines without 16-byte alignment, whose copies cost the
-// streaming warp an instruction an element, take 32 rows a warp up to 8 groups
-// an SM.  Long lines in few groups stay with the scans.
-enum LineForm { kLineScan, kLineTile16, kLineTile32, kLineTile64, kLineMarch };
+// The form of ch_march.cuh, or the scans, that solves substep l's lines of dir.
 template <typename T>
 LineForm line_form(const ch_handle* h, int l, int dir) {
-    const LineTables& lt = h->lines[dir][l];
-    const int64_t nx = h->n[0], ny = h->n[1], nz = h->n[2];
-    if (!lt.reach || lt.n < (sizeof(T) == 4 ? 65 : 64) || lt.reach > lt.n) return kLineScan;
-    const int64_t groups = dir == 0 ? (ny * nz + 31) / 32 : dir == 1 ? (nx + 31) / 32 * nz : (nx * ny + 31) / 32;
-    const int64_t row = dir == 2 ? nx * ny : nx;
-    auto fits = [&](auto rc) {
-        constexpr int R = decltype(rc)::value;
-        const int warps = tile_warps<R>(lt.n, lt.reach);
-        return warps <= tile_max_warps<R>() &&
-               std::max(tile_yz_bytes<T, R>(warps), tile_x_bytes<T, R>(warps)) <= kMaxSmem;
-    };
-    const bool fits32 = fits(std::integral_constant<int, 32>{});
-    if (sizeof(T) == 8) {
-        if (groups >= 3 * 152 && fits(std::integral_constant<int, 64>{})) return kLineTile64;
-        return fits32 ? kLineTile32 : groups >= 2 * 152 ? kLineMarch : kLineScan;
-    }
-    if (row % 4 != 0 && fits32 && groups <= 8 * 152) return kLineTile32;
-    if (groups <= 2 * 152 && tile_warps<16>(lt.n, lt.reach) <= tile_max_warps<16>()) return kLineTile16;
-    return groups >= 2 * 152 ? kLineMarch : kLineScan;
+    return choose_line_form<T>({{h->n[0], h->n[1], h->n[2]}, dir, h->p.bc[dir] == CH_PERIODIC, h->lines[dir][l].reach});
 }
 
 // Two columns per thread (paired FP32 arithmetic, 256-byte rows) while that
@@ -585,7 +544,7 @@ template <typename T>
 MarchCoef<T> march_coef(const ch_handle* h, int l, int dir) {
     const LineTables& lt = h->lines[dir][l];
     return {(T)-lt.march[0], (T)-lt.march[1], (T)lt.march[2], lt.n, h->p.bc[dir], lt.reach,
-            (lt.reach + MarchShape<T>::B - 1) / MarchShape<T>::B};
+            march_kb<T>(lt.reach)};
 }
 
 template <typename T, int V, int VL>

@@ -9,6 +9,7 @@ import pytest
 from oracle import ch_oracle as co
 from paper_2105_01865_gb300 import inputs
 
+import _line_form as lf
 from _parity import assert_parity
 
 pytestmark = pytest.mark.gpu
@@ -69,3 +70,38 @@ def test_one_step_matches_oracle(shape, ck, prec, bc=None):
     ref = co.step(C0, None, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=dt, bc=bc), 1)
     # backward-stable solves: a few roundings times the condition number of (I + ck [1,-4,6,-4,1])
     assert_parity(got, ref, 8 * (1 + 16 * ck) * 2.0 ** (-53 if prec == "f64" else -24), f"march {shape} {bc} ck={ck} {prec}")
+
+
+# boxes that take every form of the line solvers in every direction, copy width and kind of wall
+# (test_march_factors.py counts them)
+@pytest.mark.parametrize("shape, prec, ck", lf.BOXES)
+@pytest.mark.parametrize("bc", [(P, P, P), (N, N, D)])
+def test_every_form_matches_oracle(shape, prec, ck, bc):
+    test_one_step_matches_oracle(shape, ck, prec, bc)
+
+
+# FP32 boxes too large for the oracle: rows of single-element copies, and over 6080 groups of 64 columns, the last
+# one partial, which take two columns a thread; restarts of one block of 32 rows and of three
+@pytest.mark.parametrize("shape, ck", [((501, 251, 201), 0.25), ((130, 620, 628), 0.25), ((130, 620, 628), 12.0),
+                                       ((1020, 200, 324), 0.25), ((1020, 200, 324), 12.0)])
+@pytest.mark.parametrize("bc", [(P, P, P), (P, N, N), (N, P, D)])
+def test_large_boxes_match_fp64(shape, bc, ck):
+    """One step against the library's FP64 form, which the oracle pins above."""
+    from paper_2105_01865_gb300.solver import Solver
+    assert lf.forms("f32", bc, shape, ck) == ("march",) * 3
+    h, cn, pe = 1.0 / 32, 0.75 / 32, 100.0
+    dt = ck / (8.0 / 15.0 / pe / 2.0 * 4.0 * cn ** 2 / h ** 4)
+    gen = torch.Generator(device="cuda").manual_seed(shape[0])
+    C0 = torch.rand(shape, generator=gen, device="cuda", dtype=torch.float32)
+    out = {}
+    for prec in ("f64", "f32"):
+        s = Solver(shape, h, bc, cn, pe, dt, C0, precision=prec)
+        s.step(1)
+        s.sync()
+        out[prec] = s.C.double()
+        s.close()
+    d = out["f32"] - out["f64"]
+    l2, em = float(d.norm() / out["f64"].norm()), float(d.abs().max() / out["f64"].abs().max())
+    bar = 8 * (1 + 16 * ck) * 2.0 ** -24  # as above
+    print(f"{shape} {bc} ck={ck}: rel L2 {l2:.2e}, max elem {em:.2e} (bar {bar:.1e})")
+    assert l2 <= bar and em <= 10 * bar
