@@ -532,8 +532,8 @@ bool multi_line_any(const ch_handle* h, int l, int dir) {
 
 // The form of ch_march.cuh, or the scans, that solves substep l's lines of dir.
 template <typename T>
-LineForm line_form(const ch_handle* h, int l, int dir) {
-    return choose_line_form<T>({{h->n[0], h->n[1], h->n[2]}, dir, h->p.bc[dir] == CH_PERIODIC, h->lines[dir][l].reach});
+LineForm line_form(const ch_handle* h, int l, int dir, bool copied) {
+    return choose_line_form<T>({{h->n[0], h->n[1], h->n[2]}, dir, h->p.bc[dir] == CH_PERIODIC, h->lines[dir][l].reach, copied});
 }
 
 // Two columns per thread (paired FP32 arithmetic, 256-byte rows) while that
@@ -659,7 +659,7 @@ int set_attrs_march(ch_handle* h) {
 template <typename T>
 int launch_solve(ch_handle* h, int l, int dir, const T* src, T* r, T* Cupd, cudaEvent_t ev_after) {
     int rc = -1;
-    switch (line_form<T>(h, l, dir)) {
+    switch (line_form<T>(h, l, dir, src != r)) {
         case kLineMarch: rc = launch_march<T>(h, l, dir, src, r, Cupd); break;
         case kLineTile32: rc = launch_tile<T, 32>(h, l, dir, src, r, Cupd); break;
         case kLineTile64:

@@ -7,14 +7,15 @@
 // odd rows; the others pay `reach` rows of restart up and down for every chunk or
 // block, which a slowly decaying operator can make longer than the line itself.
 // So each form's time is estimated and the least taken:
-//   us = t0 + sqrt((row x rows in sequence)^2 + (work x rows in all / SM)^2 + (mem x copy time)^2)
-// (the scans have no third term).  The constants are least-squares fits to 2958
-// solves timed in every form (50 boxes of 64 x 64 x 1 to 1024 x 1024 x 128, odd and
-// even rows, periodic and walled lines of 20 to 1024 rows, every restart distance);
-// nine in ten estimates are within 15 % (FP32) and 20 % (FP64).  The form taken is on
-// average 2 % slower than the fastest; it is over 5 % slower than the scans in 18 of
-// the solves, 25 % at most (80-row walled lines, 25 against 21 us).  Thresholds on
-// groups and length, tried before, were slower than the scans in 460, up to 4.9 times.
+//   us = t0 + the 4-norm of (row x rows in sequence, work x rows in all / SM, mem x copy time)
+// (the scans have no third term).  The constants are those that lose least by the
+// choice over 7798 solves timed in every form, back to back (101 boxes of 24^3 to
+// 1024 x 512 x 128, planes among them, odd and even rows, periodic and walled lines of 24
+// to 1024 rows, seven restart distances); as times of one solve they are rough.  The form
+// taken is on average 0.5 (FP32) and 1 % (FP64) slower than the fastest, and over 10 %
+// slower than the scans in 25 of the solves, 28 % at most; most of these take 6 to 15 us,
+// where a launch moves in steps of 2 us.  Thresholds on groups and length were slower
+// than the scans by up to 4.9 times.
 #pragma once
 
 #include <cmath>
@@ -64,6 +65,7 @@ struct LineBox {
     int dir;
     bool periodic;  // along dir
     int reach;      // restart distance (0: the operator decays too slowly)
+    bool copied;    // the right-hand sides are not where the solution goes
 };
 
 // Whether a form takes the lines at all: none is shorter than its restart, and
@@ -84,9 +86,14 @@ inline int64_t line_groups(const LineBox& b) {
     return b.dir == 0 ? (b.n[1] * b.n[2] + 31) / 32 : b.dir == 1 ? (b.n[0] + 31) / 32 * b.n[2] : (b.n[0] * b.n[1] + 31) / 32;
 }
 
+inline double norm4(double a, double b, double c) { return std::sqrt(std::sqrt(a * a * a * a + b * b * b * b + c * c * c * c)); }
+
 struct ScanCost {
-    double t0, row, walled, even, odd;  // walled lines, nx = 2 mod 4 and odd: factors on the work
-    double work[6];                     // of 32-line groups, for M = 1, 2, 4, .. 32 rows a lane
+    double t0, row;
+    // factors on the work: walled lines where nx is a multiple of 4 and elsewhere;
+    // nx a multiple of 4, of 2 alone, odd
+    double walled[2], align[3];
+    double work[6];  // of 32-line groups, for M = 1, 2, 4, .. 32 rows a lane
 };
 struct MarchCost {
     double t0, row, work, mem;
@@ -94,38 +101,46 @@ struct MarchCost {
 
 template <typename T>
 double scan_us(const LineBox& b) {
-    static constexpr ScanCost k[2][3] = {
-        {{5.7, 0.19, 0.70, 1.44, 1.70, {1.19, 1.49, 1.88, 3.41, 6.93, 14.1}},
-         {7.9, 0.27, 0.77, 1.06, 1.76, {0.43, 0.76, 1.58, 4.16, 6.55, 14.4}},
-         {8.0, 0.26, 0.78, 1.06, 1.86, {0.46, 1.14, 2.07, 5.23, 7.52, 22.5}}},
-        {{15.5, 0.85, 0.80, 1.0, 1.0, {20.6, 23.4, 36.1, 58.0, 89.4, 189.0}},
-         {5.4, 7.65, 0.85, 1.0, 1.0, {11.2, 16.1, 27.9, 66.4, 179.0, 390.0}},
-         {9.3, 10.4, 0.86, 1.06, 1.06, {11.6, 17.5, 30.1, 74.5, 221.0, 480.0}}}};
+    static constexpr ScanCost k[2][3] = {{{1.71, 0.308, {0.491, 0.651}, {1.0, 1.05, 0.993}, {1.36, 2.18, 2.26, 5.03, 14.1, 34.1}},
+                                          {3.46, 0.601, {0.366, 0.629}, {1.0, 0.996, 1.5}, {0.479, 1.38, 2.7, 14.5, 13.3, 14.8}},
+                                          {2.93, 0.0155, {0.621, 0.696}, {1.0, 1.1, 2.85}, {0.622, 1.41, 3.26, 8.32, 14.7, 19.6}}},
+                                         {{5.88, 0.715, {0.906, 0.766}, {1.0, 1.06, 1.04}, {21.3, 29.8, 39.2, 60.7, 74.3, 197.0}},
+                                          {9.23, 5.43, {0.738, 0.728}, {1.0, 0.822, 0.956}, {11.2, 20.3, 36.6, 82.1, 212.0, 229.0}},
+                                          {0.0578, 9.71, {0.821, 0.927}, {1.0, 1.1, 0.936}, {12.4, 26.5, 43.5, 82.1, 194.0, 268.0}}}};
     const ScanCost& c = k[sizeof(T) == 8][b.dir];
     int m = 0;
     while ((32 << m) < b.n[b.dir]) ++m;
     const double per_sm = (double)line_groups(b) / 152.0;
-    const double align = b.n[0] % 4 == 0 ? 1.0 : b.n[0] % 2 == 0 ? c.even : c.odd;
+    const int al = b.n[0] % 4 == 0 ? 0 : b.n[0] % 2 == 0 ? 1 : 2;
+    const double work = c.work[m] * c.align[al] * (b.periodic ? 1.0 : c.walled[al > 0]);
     // over 512 rows (M = 32) other kernels, with no longer a sequence
-    return c.t0 + std::hypot(c.row * (m < 5 ? 1 << m : 16), per_sm * c.work[m] * (b.periodic ? 1.0 : c.walled) * align);
+    const double t = c.t0 + norm4(c.row * (m < 5 ? 1 << m : 16), per_sm * work, 0.0);
+    // they work in place: a launch to copy the right-hand sides first
+    return b.copied ? t + 2.0 + 2.0 * sizeof(T) * b.n[0] * b.n[1] * b.n[2] / 6.69e6 : t;
 }
 
 template <typename T>
 double march_us(const LineBox& b, LineForm f) {
-    // by form, x and y or z (which also reads and writes C)
-    static constexpr MarchCost f32[4][2] = {{{6.5, 0.055, 0.0029, 1.43}, {6.5, 0.058, 0.0033, 1.37}},
-                                            {{7.6, 0.044, 0.0034, 1.35}, {7.1, 0.064, 0.0038, 1.48}},
-                                            {{8.0, 0.0063, 0.00168, 0.33}, {8.3, 0.0081, 0.0019, 0.94}},
-                                            {{8.5, 0.0104, 0.0027, 0.0}, {9.1, 0.022, 0.0031, 1.42}}};
-    static constexpr MarchCost f64[4][2] = {{{5.7, 0.24, 0.036, 6.4}, {5.1, 0.25, 0.0375, 6.2}},
-                                            {{5.2, 0.23, 0.042, 6.6}, {6.2, 0.25, 0.046, 5.8}},
-                                            {{1.4, 0.09, 0.0335, 7.3}, {0.0, 0.11, 0.047, 3.7}},
-                                            {{8.9, 0.09, 0.038, 6.4}, {0.0, 0.11, 0.047, 3.7}}};
+    // tiles of 16 (FP64: 32) and 32 (64) rows and streams, on rows that are 16-byte
+    // aligned and that are not, along x, y and z (which also reads and writes C)
+    static constexpr MarchCost k[2][3][2][3] = {
+        {{{{2.37, 0.112, 0.00443, 1.57}, {2.74, 0.0595, 0.00508, 0.238}, {2.84, 0.0117, 0.00512, 1.57}},
+          {{0.00752, 0.179, 0.00524, 0.0869}, {2.59, 0.057, 0.00469, 1.82}, {0.0293, 0.114, 0.00648, 0.53}}},
+         {{{0.351, 0.153, 0.00557, 1.47}, {0.00442, 0.133, 0.00668, 2.81}, {3.55, 0.0973, 0.00644, 2.52}},
+          {{5.14, 0.0503, 0.00331, 0.127}, {7.19, 0.0, 0.00422, 1.54}, {0.115, 0.152, 0.00609, 0.219}}},
+         {{{0.00631, 0.0135, 0.00273, 0.0343}, {2.5, 0.00934, 0.00156, 0.0601}, {3.48, 0.011, 0.00263, 0.0468}},
+          {{8.54, 0.0157, 0.00302, 0.01}, {2.43, 0.0144, 0.00325, 0.00989}, {1.27, 0.0407, 0.00359, 0.01}}}},
+        {{{{7.48, 0.215, 0.0422, 7.99}, {0.00181, 0.286, 0.0471, 0.599}, {0.00237, 0.304, 0.0438, 7.54}},
+          {{11.8, 0.123, 0.0337, 10.5}, {0.0, 0.322, 0.0548, 0.593}, {0.00365, 0.369, 0.046, 0.572}}},
+         {{{10.8, 0.15, 0.0502, 0.532}, {4.59, 0.189, 0.0548, 0.418}, {6.97, 0.187, 0.056, 0.449}},
+          {{0.0149, 0.696, 0.00656, 8.52}, {18.0, 0.00159, 0.0529, 0.322}, {0.181, 0.0156, 0.0586, 6.71}}},
+         {{{0.00252, 0.0812, 0.0578, 0.837}, {0.0533, 0.101, 0.0481, 2.3}, {0.0544, 0.128, 0.0448, 12.0}},
+          {{0.0, 0.0763, 0.0418, 1.23}, {0.0, 0.0879, 0.0454, 12.1}, {2.05, 0.106, 0.0468, 13.4}}}}};
     const int z = b.dir == 2, n = (int)b.n[b.dir];
     const int64_t row = z ? b.n[0] * b.n[1] : b.n[0];  // columns of a row of lines: its alignment
     const bool aligned = row * sizeof(T) % 16 == 0;
-    const MarchCost& c = sizeof(T) == 8 ? f64[f == kLineTile32 ? 0 : f == kLineTile64 ? 1 : aligned ? 2 : 3][z]
-                                        : f32[f == kLineTile16 ? 0 : f == kLineTile32 ? 1 : aligned ? 2 : 3][z];
+    const int form = f == kLineMarch ? 2 : f == (sizeof(T) == 8 ? kLineTile32 : kLineTile16) ? 0 : 1;
+    const MarchCost& c = k[sizeof(T) == 8][form][!aligned][b.dir];
     double seq, all;  // rows in sequence, and in all of a line
     if (f == kLineMarch) {
         const int B = MarchShape<T>::B, kb = march_kb<T>(b.reach), nb = (n + B - 1) / B;
@@ -137,17 +152,13 @@ double march_us(const LineBox& b, LineForm f) {
     }
     const double groups = (double)line_groups(b);
     const double copy = groups * 32.0 * n * sizeof(T) * (z ? 3 : 2) / 6.69e6;  // us at 6.69 TB/s
-    const double w = c.work * all * groups / 152.0;
-    return c.t0 + std::sqrt(c.row * seq * c.row * seq + w * w + c.mem * copy * c.mem * copy);
+    return c.t0 + norm4(c.row * seq, c.work * all * groups / 152.0, c.mem * copy);
 }
 
 template <typename T>
 LineForm choose_line_form(const LineBox& b) {
-    // FP64 x-lines of a plane, in a few warps: the fit is too high there (18 us in the
-    // scan, 29 in a tile, for 256 lines of 256 rows)
-    if (sizeof(T) == 8 && b.dir == 0 && line_groups(b) <= 16) return kLineScan;
     LineForm best = kLineScan;
-    double least = 0.9 * scan_us<T>(b);  // the estimates' spread: leave the scans for a clear gain
+    double least = scan_us<T>(b);
     auto consider = [&](LineForm f, bool fits) {
         const double t = fits ? march_us<T>(b, f) : least;
         if (t < least) {

@@ -27,20 +27,18 @@ static int query(const LineBox& b, double* us) {
     return choose_line_form<T>(b);
 }
 extern "C" int form(int fp64, int periodic, int dir, long nx, long ny, long nz, int reach, double* us) {
-    const LineBox b{{nx, ny, nz}, dir, periodic != 0, reach};
+    const LineBox b{{nx, ny, nz}, dir, periodic != 0, reach, false};
     return fp64 ? query<double>(b, us) : query<float>(b, us);
 }
 """
 # (nz, ny, nx), precision and ck of boxes that take every form
-BOXES = [((500, 64, 48), "f32", 0.25), ((300, 96, 36), "f32", 0.25), ((64, 48, 501), "f32", 0.25), ((34, 33, 257), "f32", 0.02),
-         ((72, 40, 260), "f32", 0.02), ((97, 34, 301), "f32", 0.25), ((33, 65, 33), "f32", 0.02), ((64, 65, 36), "f32", 0.02),
-         ((33, 300, 33), "f32", 0.25), ((33, 300, 36), "f32", 0.25), ((33, 126, 33), "f32", 0.02), ((65, 40, 33), "f32", 0.02),
-         ((300, 33, 33), "f32", 0.25), ((300, 34, 34), "f32", 0.25), ((128, 34, 300), "f32", 0.25),
-         ((48, 33, 33), "f64", 0.02), ((48, 33, 34), "f64", 0.02), ((126, 48, 97), "f64", 1.2), ((126, 48, 96), "f64", 1.2),
-         ((72, 500, 33), "f64", 0.02), ((64, 500, 34), "f64", 0.02), ((33, 33, 34), "f64", 0.02), ((33, 34, 33), "f64", 0.02),
-         ((72, 160, 33), "f64", 1.2), ((72, 160, 34), "f64", 1.2), ((500, 97, 33), "f64", 0.02), ((500, 40, 70), "f64", 0.02),
-         ((96, 129, 65), "f64", 1.2), ((96, 126, 65), "f64", 1.2), ((102, 500, 66), "f64", 3.0), ((500, 99, 99), "f64", 3.0),
-         ((98, 100, 520), "f64", 0.25), ((98, 100, 517), "f64", 0.25)]
+BOXES = [((33, 36, 33), "f32", 0.02), ((33, 33, 36), "f32", 0.02), ((65, 33, 33), "f32", 0.02), ((33, 33, 260), "f32", 0.02),
+         ((200, 40, 36), "f32", 0.25), ((400, 48, 33), "f32", 0.25), ((300, 33, 33), "f32", 0.25), ((33, 300, 33), "f32", 0.25),
+         ((33, 300, 36), "f32", 0.25), ((64, 48, 301), "f32", 0.25), ((72, 67, 300), "f32", 0.25),
+         ((33, 33, 33), "f64", 0.02), ((33, 33, 34), "f64", 0.02), ((66, 40, 33), "f64", 0.02), ((72, 34, 36), "f64", 0.02),
+         ((70, 501, 33), "f64", 0.02), ((97, 500, 34), "f64", 0.02), ((500, 65, 65), "f64", 0.02), ((500, 72, 70), "f64", 0.02),
+         ((500, 97, 65), "f64", 0.02), ((500, 97, 65), "f64", 3.0), ((33, 72, 33), "f64", 1.2), ((36, 104, 96), "f64", 1.2),
+         ((96, 160, 36), "f64", 1.2), ((98, 100, 520), "f64", 0.25), ((98, 100, 517), "f64", 0.25)]
 NAMES = ("scan", "tile16", "tile32", "tile64", "march")
 _lib = None
 
