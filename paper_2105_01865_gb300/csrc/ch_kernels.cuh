@@ -160,7 +160,9 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // Explicitly rounded multiply-adds: the solver's arithmetic is fixed in the
 // source, so every kernel that inlines it (standalone, batched persistent,
-// batched per phase) rounds identically and the results agree bit for bit.
+// batched per phase) rounds identically and the results agree bit for bit.  (A
+// line that a single box gives to a form of ch_march.cuh, and the batch to this
+// solver, agrees to rounding.)
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }

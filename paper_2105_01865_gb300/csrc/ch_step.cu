@@ -724,9 +724,9 @@ int set_attrs_m(ch_handle* h) {
 // diffusive or implicit term, no right-hand side written.
 // Planes a tile marches: the depth whose waves of CTAs take the least, a tile
 // costing its planes and about kTileStart more (its z-queue and first copies).
-// Against fixed depths: 256 x 256 x 128, 91 us (19 planes) and 92 (16) or 114
-// (64); 500^3, 1211 us (56) and 1333 (64); 64^3 without advection, 7 us (2)
-// and 11 (10); 1024 x 1024 x 512, 4.85 ms either way (64).
+// Against fixed depths: 256 x 256 x 128, 88 us (19 planes) and 87 (16) or 105
+// (64); 500^3, 1134 us (56) and 1141 (64); 64^3 without advection, 6.6 us (2)
+// and 9.0 (10); 1024 x 1024 x 512, 4.60 ms (256) and as much (64).
 inline int explicit_depth(int64_t xy, int nz, int64_t slots) {
     constexpr double kTileStart = 2.0;
     int best = nz;
@@ -783,11 +783,11 @@ int launch_explicit(ch_handle* h, int l, const T* C, const T* Hprev, T* Hout, T*
     if (ev) CHG_CUDA(h, cudaEventRecord(ev[0], h->stream));
     if constexpr (sizeof(T) == 8) {
         const bool diri = p.bc[2] == CH_DIRICHLET;
-        // 8-row tiles, 3 CTAs an SM: 2757 us on the 256 x 256 x 128 shear drop,
-        // 2835 with 2 CTAs, 2913 with 16-row tiles (1 CTA: every warp meets at
-        // the same barriers).  A z-chunk costs about half a plane to start:
-        // 16 planes, halved while that leaves fewer than 6 CTAs an SM (64^3: 91
-        // us with 56 CTAs of 10 planes, 35 with 512 of 2).
+        // 8-row tiles, 3 CTAs an SM (2 were 3 % slower on the 256 x 256 x 128 shear
+        // drop, 16-row tiles, 1 CTA whose warps all meet at the same barriers, 6 %).
+        // A z-chunk costs about half a plane to start: 16 planes (2587 us there; 32:
+        // 2575, 8: 2553), halved while that leaves fewer than 6 CTAs an SM (64^3
+        // without advection: 63 us in chunks of 16 planes, 35 in its 2).
         constexpr int TY = 8, MINB = 3;
         const int64_t xy = (int64_t)((nx + kEX - 1) / kEX) * ((ny + TY - 1) / TY);
         int tz = 16;

@@ -158,3 +158,26 @@ def test_batch_64_uneven_boxes():
     for i in (0, 17, 63):
         ref = single(boxes[i], 3)
         assert np.abs(got[i] - ref).max() <= 1e-6 * np.abs(ref).max()
+
+
+# lines that a single box gives to the marching solvers and the batch to the scans, walled and unaligned rows
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("bc", [(0, 0, 0), (1, 0, 1), (1, 1, 1)])
+def test_longer_lines_agree_with_single_box_runs(mode, bc):
+    from paper_2105_01865_gb300.solver import Batch
+    boxes = []
+    rng = np.random.default_rng(21)
+    for n in ((66, 70, 30), (96, 96, 96), (90, 34, 128), (128, 66, 20)):
+        h = 1.0 / max(n)
+        cn, pe = 0.75 * h, 500.0
+        C = inputs.drops_field(n, h, bc, [(n[2] * h * 0.5, n[1] * h * 0.45, n[0] * h * 0.55)], [0.3 * min(n) * h], cn)
+        boxes.append(dict(shape=n, h=h, bc=bc, cn=cn, pe=pe, C=C + 0.02 * rng.standard_normal(n),
+                          dt=0.9 * stability.stable_dt(n, h, bc, cn, pe, max_modes=12)))
+    b = Batch(boxes)
+    b.set_schedule(mode, 3, 8, 1)
+    b.step(3)
+    got = b.fields()
+    b.close()
+    for box, g in zip(boxes, got):
+        ref = single(box, 3)
+        assert np.abs(g - ref).max() <= 1e-6 * np.abs(ref).max(), box["shape"]  # the bar of the tests above
