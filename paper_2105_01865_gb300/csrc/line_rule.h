@@ -9,13 +9,13 @@
 // So each form's time is estimated and the least taken:
 //   us = t0 + the 4-norm of (row x rows in sequence, work x rows in all / SM, mem x copy time)
 // (the scans have no third term).  The constants are those that lose least by the
-// choice over 7798 solves timed in every form, back to back (101 boxes of 24^3 to
-// 1024 x 512 x 128, planes among them, odd and even rows, periodic and walled lines of 24
-// to 1024 rows, seven restart distances); as times of one solve they are rough.  The form
-// taken is on average 0.5 (FP32) and 1 % (FP64) slower than the fastest, and over 10 %
-// slower than the scans in 25 of the solves, 28 % at most; most of these take 6 to 15 us,
-// where a launch moves in steps of 2 us.  Thresholds on groups and length were slower
-// than the scans by up to 4.9 times.
+// choice over 14538 solves timed in every form, back to back (216 boxes of 8^3 to
+// 1024 x 1024 x 512, planes among them, odd and even rows, periodic and walled lines,
+// restarts of 8 to 96 rows); as times of one solve they are rough.  The form taken is on
+// average 0.4 (FP32) and 0.9 % (FP64) slower than the fastest, and over 10 % slower than
+// the scans in 58 of the solves, 44 % at most; most of these take 4 to 15 us, where a
+// launch moves in steps of 2 us.  Thresholds on groups and length were slower than the
+// scans by up to 4.9 times.
 #pragma once
 
 #include <cmath>
@@ -89,7 +89,7 @@ inline int64_t line_groups(const LineBox& b) {
 inline double norm4(double a, double b, double c) { return std::sqrt(std::sqrt(a * a * a * a + b * b * b * b + c * c * c * c)); }
 
 struct ScanCost {
-    double t0, row;
+    double t0[2], row;  // t0 of periodic and of walled lines
     // factors on the work: walled lines where nx is a multiple of 4 and elsewhere;
     // nx a multiple of 4, of 2 alone, odd
     double walled[2], align[3];
@@ -101,12 +101,12 @@ struct MarchCost {
 
 template <typename T>
 double scan_us(const LineBox& b) {
-    static constexpr ScanCost k[2][3] = {{{1.71, 0.308, {0.491, 0.651}, {1.0, 1.05, 0.993}, {1.36, 2.18, 2.26, 5.03, 14.1, 34.1}},
-                                          {3.46, 0.601, {0.366, 0.629}, {1.0, 0.996, 1.5}, {0.479, 1.38, 2.7, 14.5, 13.3, 14.8}},
-                                          {2.93, 0.0155, {0.621, 0.696}, {1.0, 1.1, 2.85}, {0.622, 1.41, 3.26, 8.32, 14.7, 19.6}}},
-                                         {{5.88, 0.715, {0.906, 0.766}, {1.0, 1.06, 1.04}, {21.3, 29.8, 39.2, 60.7, 74.3, 197.0}},
-                                          {9.23, 5.43, {0.738, 0.728}, {1.0, 0.822, 0.956}, {11.2, 20.3, 36.6, 82.1, 212.0, 229.0}},
-                                          {0.0578, 9.71, {0.821, 0.927}, {1.0, 1.1, 0.936}, {12.4, 26.5, 43.5, 82.1, 194.0, 268.0}}}};
+    static constexpr ScanCost k[2][3] = {{{{3.05, 4.1}, 0.19, {0.441, 0.566}, {1.0, 0.893, 1.19}, {0.883, 1.49, 2.27, 4.51, 11.9, 30.2}},
+                                          {{5.5, 4.11}, 0.628, {0.732, 0.835}, {1.0, 1.2, 1.97}, {0.285, 0.632, 1.5, 5.6, 6.83, 24.0}},
+                                          {{4.73, 3.55}, 0.924, {0.766, 0.87}, {1.0, 1.36, 3.11}, {0.308, 0.999, 2.3, 6.31, 11.0, 22.4}}},
+                                         {{{11.1, 6.72}, 0.372, {1.01, 0.94}, {1.0, 1.9, 1.15}, {21.9, 30.1, 33.6, 53.4, 74.5, 145.0}},
+                                          {{10.4, 4.15}, 6.98, {0.942, 0.963}, {1.0, 0.902, 0.826}, {12.7, 17.2, 36.1, 73.3, 187.0, 177.0}},
+                                          {{6.29, 2.87}, 8.61, {0.98, 1.0}, {1.0, 1.01, 0.998}, {13.0, 22.4, 38.2, 73.3, 187.0, 211.0}}}};
     const ScanCost& c = k[sizeof(T) == 8][b.dir];
     int m = 0;
     while ((32 << m) < b.n[b.dir]) ++m;
@@ -114,7 +114,7 @@ double scan_us(const LineBox& b) {
     const int al = b.n[0] % 4 == 0 ? 0 : b.n[0] % 2 == 0 ? 1 : 2;
     const double work = c.work[m] * c.align[al] * (b.periodic ? 1.0 : c.walled[al > 0]);
     // over 512 rows (M = 32) other kernels, with no longer a sequence
-    const double t = c.t0 + norm4(c.row * (m < 5 ? 1 << m : 16), per_sm * work, 0.0);
+    const double t = c.t0[!b.periodic] + norm4(c.row * (m < 5 ? 1 << m : 16), per_sm * work, 0.0);
     // they work in place: a launch to copy the right-hand sides first
     return b.copied ? t + 2.0 + 2.0 * sizeof(T) * b.n[0] * b.n[1] * b.n[2] / 6.69e6 : t;
 }
@@ -124,18 +124,18 @@ double march_us(const LineBox& b, LineForm f) {
     // tiles of 16 (FP64: 32) and 32 (64) rows and streams, on rows that are 16-byte
     // aligned and that are not, along x, y and z (which also reads and writes C)
     static constexpr MarchCost k[2][3][2][3] = {
-        {{{{2.37, 0.112, 0.00443, 1.57}, {2.74, 0.0595, 0.00508, 0.238}, {2.84, 0.0117, 0.00512, 1.57}},
-          {{0.00752, 0.179, 0.00524, 0.0869}, {2.59, 0.057, 0.00469, 1.82}, {0.0293, 0.114, 0.00648, 0.53}}},
-         {{{0.351, 0.153, 0.00557, 1.47}, {0.00442, 0.133, 0.00668, 2.81}, {3.55, 0.0973, 0.00644, 2.52}},
-          {{5.14, 0.0503, 0.00331, 0.127}, {7.19, 0.0, 0.00422, 1.54}, {0.115, 0.152, 0.00609, 0.219}}},
-         {{{0.00631, 0.0135, 0.00273, 0.0343}, {2.5, 0.00934, 0.00156, 0.0601}, {3.48, 0.011, 0.00263, 0.0468}},
-          {{8.54, 0.0157, 0.00302, 0.01}, {2.43, 0.0144, 0.00325, 0.00989}, {1.27, 0.0407, 0.00359, 0.01}}}},
-        {{{{7.48, 0.215, 0.0422, 7.99}, {0.00181, 0.286, 0.0471, 0.599}, {0.00237, 0.304, 0.0438, 7.54}},
-          {{11.8, 0.123, 0.0337, 10.5}, {0.0, 0.322, 0.0548, 0.593}, {0.00365, 0.369, 0.046, 0.572}}},
-         {{{10.8, 0.15, 0.0502, 0.532}, {4.59, 0.189, 0.0548, 0.418}, {6.97, 0.187, 0.056, 0.449}},
-          {{0.0149, 0.696, 0.00656, 8.52}, {18.0, 0.00159, 0.0529, 0.322}, {0.181, 0.0156, 0.0586, 6.71}}},
-         {{{0.00252, 0.0812, 0.0578, 0.837}, {0.0533, 0.101, 0.0481, 2.3}, {0.0544, 0.128, 0.0448, 12.0}},
-          {{0.0, 0.0763, 0.0418, 1.23}, {0.0, 0.0879, 0.0454, 12.1}, {2.05, 0.106, 0.0468, 13.4}}}}};
+        {{{{4.12, 0.085, 0.00348, 1.51}, {3.49, 0.0694, 0.00487, 0.149}, {2.67, 0.0801, 0.00435, 1.61}},
+          {{4.68, 0.0718, 0.00419, 0.0743}, {3.74, 0.0601, 0.00395, 1.48}, {2.45, 0.0733, 0.00582, 1.55}}},
+         {{{3.56, 0.102, 0.00417, 1.26}, {0.875, 0.134, 0.00575, 2.81}, {1.56, 0.182, 0.0059, 2.71}},
+          {{6.76, 0.0504, 0.00341, 1.11}, {4.99, 0.0753, 0.00385, 1.74}, {3.99, 0.0999, 0.00552, 0.0903}}},
+         {{{3.54, 0.00921, 0.00212, 0.0157}, {3.85, 0.00847, 0.00154, 0.0289}, {3.29, 0.0115, 0.00241, 0.0302}},
+          {{4.64, 0.021, 0.00255, 0.00989}, {4.18, 0.0108, 0.00246, 0.00957}, {3.38, 0.0336, 0.00492, 0.0101}}}},
+        {{{{14.1, 0.129, 0.0393, 5.85}, {0.0, 0.293, 0.0447, 0.185}, {0.00166, 0.329, 0.0458, 3.51}},
+          {{0.0, 0.357, 0.0378, 6.57}, {6.11, 0.198, 0.0508, 0.267}, {10.8, 0.0489, 0.0421, 0.296}}},
+         {{{17.0, 0.0992, 0.0431, 3.51}, {3.26, 0.206, 0.053, 0.94}, {6.07, 0.216, 0.0561, 0.239}},
+          {{6.62, 0.202, 0.0452, 0.243}, {19.0, 0.0107, 0.0529, 0.218}, {4.14, 0.264, 0.0559, 5.95}}},
+         {{{13.2, 0.0707, 0.0383, 0.209}, {0.0, 0.104, 0.0447, 0.273}, {0.0, 0.126, 0.054, 0.483}},
+          {{11.9, 0.081, 0.0451, 1.06}, {0.0, 0.0907, 0.0456, 12.4}, {0.0, 0.124, 0.0486, 0.196}}}}};
     const int z = b.dir == 2, n = (int)b.n[b.dir];
     const int64_t row = z ? b.n[0] * b.n[1] : b.n[0];  // columns of a row of lines: its alignment
     const bool aligned = row * sizeof(T) % 16 == 0;

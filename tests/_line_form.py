@@ -32,13 +32,16 @@ extern "C" int form(int fp64, int periodic, int dir, long nx, long ny, long nz, 
 }
 """
 # (nz, ny, nx), precision and ck of boxes that take every form
-BOXES = [((33, 36, 33), "f32", 0.02), ((33, 33, 36), "f32", 0.02), ((65, 33, 33), "f32", 0.02), ((33, 33, 260), "f32", 0.02),
-         ((200, 40, 36), "f32", 0.25), ((400, 48, 33), "f32", 0.25), ((300, 33, 33), "f32", 0.25), ((33, 300, 33), "f32", 0.25),
-         ((33, 300, 36), "f32", 0.25), ((64, 48, 301), "f32", 0.25), ((72, 67, 300), "f32", 0.25),
-         ((33, 33, 33), "f64", 0.02), ((33, 33, 34), "f64", 0.02), ((66, 40, 33), "f64", 0.02), ((72, 34, 36), "f64", 0.02),
-         ((70, 501, 33), "f64", 0.02), ((97, 500, 34), "f64", 0.02), ((500, 65, 65), "f64", 0.02), ((500, 72, 70), "f64", 0.02),
-         ((500, 97, 65), "f64", 0.02), ((500, 97, 65), "f64", 3.0), ((33, 72, 33), "f64", 1.2), ((36, 104, 96), "f64", 1.2),
-         ((96, 160, 36), "f64", 1.2), ((98, 100, 520), "f64", 0.25), ((98, 100, 517), "f64", 0.25)]
+BOXES = [((33, 33, 33), "f32", 0.02), ((33, 33, 36), "f32", 0.02), ((33, 65, 36), "f32", 0.02), ((36, 33, 257), "f32", 0.02),
+         ((40, 34, 260), "f32", 0.02), ((400, 36, 36), "f32", 0.02), ((300, 33, 33), "f32", 0.25), ((33, 300, 33), "f32", 0.25),
+         ((33, 300, 36), "f32", 0.25), ((64, 64, 301), "f32", 0.25), ((72, 66, 300), "f32", 0.25),
+         ((40, 33, 33), "f64", 0.02), ((40, 33, 34), "f64", 0.02), ((64, 33, 33), "f64", 0.02), ((70, 500, 33), "f64", 0.02),
+         ((70, 500, 36), "f64", 0.02), ((500, 40, 129), "f64", 0.02), ((500, 97, 65), "f64", 0.02), ((500, 97, 65), "f64", 3.0),
+         ((96, 72, 72), "f64", 1.2), ((72, 97, 97), "f64", 1.2), ((70, 160, 33), "f64", 1.2), ((98, 100, 520), "f64", 0.25),
+         ((98, 100, 517), "f64", 0.25),
+         # lines as short as their restart
+         ((200, 200, 8), "f32", 1e-4), ((128, 8, 33), "f32", 1e-4), ((8, 32, 32), "f32", 1e-4), ((128, 32, 16), "f64", 1e-4),
+         ((128, 16, 32), "f64", 1e-4), ((16, 128, 32), "f64", 1e-4)]
 NAMES = ("scan", "tile16", "tile32", "tile64", "march")
 _lib = None
 
