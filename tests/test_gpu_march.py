@@ -105,3 +105,30 @@ def test_large_boxes_match_fp64(shape, bc, ck):
     bar = 8 * (1 + 16 * ck) * 2.0 ** -24  # as above
     print(f"{shape} {bc} ck={ck}: rel L2 {l2:.2e}, max elem {em:.2e} (bar {bar:.1e})")
     assert l2 <= bar and em <= 10 * bar
+
+
+# an operator that decays too slowly to restart, on a smooth field (whose small differences FP32 keeps): the
+# scan and column solvers of 65- to 256-row lines, even and odd rows, which other boxes of these sizes no longer take
+# (FP64 also with Dirichlet walls, next to which such a field changes by more than itself)
+@pytest.mark.parametrize("shape", [(90, 100, 66), (150, 200, 34), (66, 250, 72), (70, 130, 67)])
+@pytest.mark.parametrize("prec, bc", [("f64", (P, P, P)), ("f64", (P, P, N)), ("f64", (N, N, D)), ("f32", (P, P, P)),
+                                      ("f32", (P, P, N))])
+def test_scan_solvers_match_oracle(shape, bc, prec):
+    from paper_2105_01865_gb300.solver import Solver
+    ck = 60.0
+    assert lf.forms(prec, bc, shape, ck) == ("scan",) * 3
+    nz, ny, nx = shape
+    h, cn, pe = 1.0 / 32, 0.75 / 32, 1e4
+    dt = ck / (8.0 / 15.0 / pe / 2.0 * 4.0 * cn ** 2 / h ** 4)
+    x, y, z = ((np.arange(n) + 0.5) * 2 * np.pi / n for n in (nx, ny, nz))
+    C0 = 0.5 + 0.2 * np.cos(z)[:, None, None] * np.cos(2 * y)[None, :, None] * np.cos(x)[None, None, :]
+    if bc[2] == D:
+        C0 = (C0 - 0.5) * np.sin(z / 2)[:, None, None]
+    C0 = C0.astype(np.float32).astype(np.float64)
+    s = Solver(shape, h, bc, cn, pe, dt, C0, precision=prec)
+    s.step(1)
+    got = s.field()
+    s.close()
+    ref = co.step(C0, None, co.Params(nx, ny, nz, h, cn=cn, pe=pe, dt=dt, bc=bc), 1)
+    # the bars of the other tests of the line solvers
+    assert_parity(got, ref, 1e-12 if prec == "f64" else 1e-6, f"scans {shape} {bc} {prec}")
